@@ -12,65 +12,105 @@
 namespace octmc {
 namespace {
 
-// The data-term computation of output A-scan p by one warp (base and frac:
-// the coordinate split of its 6 displacement values); the value of this
-// lane's output (see data_core).
+// Eq. 4 (or squared differences) of a residual and its derivative.  The
+// pseudo-Huber loss is evaluated as (R^2/eps) / (1 + sqrt(1 + (R/eps)^2)): no
+// cancellation near 0.  Its arguments are never subnormal (1 + x^2 >= 1), so
+// the flush-to-zero forms of the reciprocal square root and the division give
+// the same results without the scaling of subnormals.
+__device__ __forceinline__ float rsqrt_ge1(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float div_ge1(float a, float b) {
+  float y;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+__device__ __forceinline__ void loss_grad(float R, float inv_eps, bool ssd, float* Lv, float* dL) {
+  if (ssd) {
+    *Lv = R * R;
+    *dL = 2.0f * R;
+  } else {
+    const float rr = R * inv_eps;
+    const float qv = fmaf(rr, rr, 1.0f);
+    const float is = rsqrt_ge1(qv);
+    *dL = rr * is;
+    *Lv = div_ge1(R * rr, fmaf(qv, is, 1.0f));
+  }
+}
+
+// Totals over the warp of 8 per-lane values: lane 4 v + x ends with the total
+// of value v.  The lanes are paired as in a butterfly (16, 8, 4, 2, 1), but
+// each of the first three stages keeps half of the values, so 9 shuffles do
+// the work of 40; the sums are those of a butterfly per value.
+__device__ __forceinline__ float warp_totals8(float v[8], int lane) {
+#pragma unroll
+  for (int n = 4; n >= 1; n >>= 1) {
+    const bool up = (lane & (4 * n)) != 0;
+#pragma unroll
+    for (int k = 0; k < n; k++) {
+      const float send = up ? v[k] : v[k + n];
+      const float keep = up ? v[k + n] : v[k];
+      v[k] = keep + __shfl_xor_sync(kFull, send, 4 * n);
+    }
+  }
+  float t = v[0];
+  t += __shfl_xor_sync(kFull, t, 2);
+  t += __shfl_xor_sync(kFull, t, 1);
+  return t;
+}
+
+// The data-term computation of output A-scan p (i, j) by one warp, with `tab`
+// (2 entries) the warp's shared-memory table.  Lane 4 v returns output v: v = 0 the
+// structural term, v = 1 + 3 V + c the gradient component c of scan V; lane
+// 28 the angiographic term.
 template <typename T>
-__device__ __forceinline__ float data_value(const DataArgs& A, int64_t p, int lane, const int base[6],
-                                            const float frac[6]) {
+__device__ __forceinline__ float data_value(const DataArgs& A, VolTab* tab, int64_t p, int i, int j, int lane) {
   const LevelDev& L = A.L;
   Vol VX, VY;
-  setup_vol(VX, L.sx, L, base, frac);
-  setup_vol(VY, L.sy, L, base + 3, frac + 3);
+  setup_pair(VX, VY, tab, A.disp, (int64_t)L.w * L.h, p, i, j, L, lane);
 
   const float inv_eps = 1.0f / A.eps_h;
   const bool ssd = (A.loss == OCTMC_LOSS_SSD);
-  float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  const int nst = (L.d + kOutPerIter - 1) / kOutPerIter;
-  for (int s = 0; s < nst; s++) {
-    const int kb = s * kOutPerIter;
-    float IX[4], IzX[4], IxX[4], IyX[4], IY[4], IzY[4], IxY[4], IyY[4];
-    sample_block<T>(VX, kb, lane, L.dp, IX, IzX, IxX, IyX);
-    sample_block<T>(VY, kb, lane, L.dp, IY, IzY, IxY, IyY);
-    if (lane >= 1 && lane <= kOutLanes) {
+  // L, then the x, y, z sums of dL dI for X and for Y
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  // outputs inside the volume from this lane's first output on (none for the halo lanes)
+  int left = (lane >= 1 && lane <= kOutLanes) ? L.d - 4 * (lane - 1) : 0;
+  for (int kb = 0; kb < L.d; kb += kOutPerIter, left -= kOutPerIter) {
+    float2 XZ[4], XG[4], YZ[4], YG[4];
+    sample_block<T>(VX, kb, lane, L.dp, XZ, XG);
+    sample_block<T>(VY, kb, lane, L.dp, YZ, YG);
+    auto add = [&](int o) {
+      float Lv, dL;
+      loss_grad(XZ[o].x - YZ[o].x, inv_eps, ssd, &Lv, &dL);
+      acc[0] += Lv;
+      float2 t = ffma2(both(dL), XG[o], make_float2(acc[1], acc[2]));
+      acc[1] = t.x; acc[2] = t.y;
+      acc[3] = fmaf(dL, XZ[o].y, acc[3]);
+      t = ffma2(both(dL), YG[o], make_float2(acc[4], acc[5]));
+      acc[4] = t.x; acc[5] = t.y;
+      acc[6] = fmaf(dL, YZ[o].y, acc[6]);
+    };
+    // outputs outside the volume add nothing, whatever their lanes hold
+    if (left >= 4) {
 #pragma unroll
-      for (int o = 0; o < 4; o++) {
-        const int k = kb + 4 * (lane - 1) + o;
-        if (k < L.d) {
-          const float R = IX[o] - IY[o];
-          float Lv, dL;
-          if (ssd) {
-            Lv = R * R;
-            dL = 2.0f * R;
-          } else {
-            // Eq. 4 as (R^2/eps) / (1 + sqrt(1 + (R/eps)^2)): no cancellation near 0
-            const float rr = R * inv_eps;
-            const float qv = fmaf(rr, rr, 1.0f);
-            const float is = rsqrtf(qv);
-            dL = rr * is;
-            Lv = __fdividef(R * rr, fmaf(qv, is, 1.0f));
-          }
-          acc[0] += Lv;
-          const float2 d2 = make_float2(dL, dL);
-          float2 t = ffma2(d2, make_float2(IxX[o], IyX[o]), make_float2(acc[1], acc[2]));
-          acc[1] = t.x; acc[2] = t.y;
-          t = ffma2(d2, make_float2(IzX[o], IxY[o]), make_float2(acc[3], acc[4]));
-          acc[3] = t.x; acc[4] = t.y;
-          t = ffma2(d2, make_float2(IyY[o], IzY[o]), make_float2(acc[5], acc[6]));
-          acc[5] = t.x; acc[6] = t.y;
-        }
-      }
+      for (int o = 0; o < 4; o++) add(o);
+    } else if (left > 0) {
+      add(0);
+      if (left > 1) add(1);
+      if (left > 2) add(2);
     }
   }
-#pragma unroll
-  for (int c = 0; c < 7; c++) acc[c] = warp_sum(acc[c]);
+  const float tot = warp_totals8(acc, lane);
+  const float Lsum = __shfl_sync(kFull, tot, 0);
 
   // ---- per-A-scan scalars (Eq. 6-8), float, every lane
   // Eq. 7: X validity along y at j + dy^X, Y validity along x at i + dx^Y,
   // by the zero-tangent Hermite interpolant (no overshoot: 0 <= delta <= delta_0)
   float vtx = 1.f, dvtx = 0.f, vty = 1.f, dvty = 0.f;
-  if (L.vx) validity_hermite(L.vx, L.h, VX.by, frac[1], &vtx, &dvtx);
-  if (L.vy) validity_hermite(L.vy, L.w, VY.bx, frac[3], &vty, &dvty);
+  if (L.vx) validity_hermite(L.vx, L.h, VX.by, VX.ts, &vtx, &dvtx);
+  if (L.vy) validity_hermite(L.vy, L.w, VY.bx, VY.ts, &vty, &dvty);
   const float delta0 = (float)A.delta0;
   const float delta = delta0 * vtx * vty;  // Eq. 8
   const float d = (float)L.d;
@@ -82,14 +122,8 @@ __device__ __forceinline__ float data_value(const DataArgs& A, int64_t p, int la
     const bool isX = lane < 16;
     const float* img = isX ? L.ax : L.ay;
     const int a = lane & 3, b = (lane >> 2) & 3;
-    float wa = 0.f, dwa = 0.f, wb = 0.f, dwb = 0.f;
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const float wxq = isX ? VX.wx[q] : VY.wx[q], dwxq = isX ? VX.dwx[q] : VY.dwx[q];
-      const float wyq = isX ? VX.wy[q] : VY.wy[q], dwyq = isX ? VX.dwy[q] : VY.dwy[q];
-      if (a == q) { wa = wxq; dwa = dwxq; }
-      if (b == q) { wb = wyq; dwb = dwyq; }
-    }
+    const VolTab& S = tab[isX ? 0 : 1];
+    const float wa = S.wx[a].y, dwa = S.wx[a].x, wb = S.wy[b].x, dwb = S.wy[b].y;
     const int bxs = isX ? VX.bx : VY.bx, bys = isX ? VX.by : VY.by;
     const float sv = img[(int64_t)clampi(bys - 1 + b, L.h) * L.w + clampi(bxs - 1 + a, L.w)];
     float v = wa * wb * sv, vx = dwa * wb * sv, vy = wa * dwb * sv;
@@ -105,60 +139,37 @@ __device__ __forceinline__ float data_value(const DataArgs& A, int64_t p, int la
     const float AX = (lane < 16) ? v : ov, AY = (lane < 16) ? ov : v;
     aXx = (lane < 16) ? vx : ovx; aXy = (lane < 16) ? vy : ovy;
     aYx = (lane < 16) ? ovx : vx; aYy = (lane < 16) ? ovy : vy;
-    const float Ra = AX - AY;
-    if (ssd) {
-      La = Ra * Ra;
-      dLa = 2.0f * Ra;
-    } else {
-      const float rr = Ra * inv_eps;
-      const float qv = fmaf(rr, rr, 1.0f);
-      const float is = rsqrtf(qv);
-      dLa = rr * is;
-      La = __fdividef(Ra * rr, fmaf(qv, is, 1.0f));
-    }
+    loss_grad(AX - AY, inv_eps, ssd, &La, &dLa);
   }
 
-  // eight outputs of this A-scan, one per lane 0..7
   const float eta = (float)(A.eta_dev ? *A.eta_dev : A.eta);
-  const float Lsum = acc[0];
   const float cs = eta * (1.0f - delta);
   const float ca = delta * d / eta * dLa;
   const float ddelta = -eta * Lsum + d * La / eta;
   float out;
-  switch (lane) {
+  switch (lane >> 2) {
     case 0: out = (1.0f - delta) * Lsum; break;
-    case 1: out = delta * d * La; break;
-    case 2: out = cs * acc[1] + ca * aXx; break;
-    case 3: out = cs * acc[2] + ca * aXy + ddelta * delta0 * dvtx * vty; break;
-    case 4: out = cs * acc[3]; break;
-    case 5: out = -cs * acc[4] - ca * aYx + ddelta * delta0 * vtx * dvty; break;
-    case 6: out = -cs * acc[5] - ca * aYy; break;
-    default: out = -cs * acc[6]; break;
+    case 1: out = fmaf(ca, aXx, cs * tot); break;
+    case 2: out = fmaf(ddelta * delta0 * dvtx, vty, fmaf(ca, aXy, cs * tot)); break;
+    case 3: out = cs * tot; break;
+    case 4: out = fmaf(ddelta * delta0 * vtx, dvty, fmaf(-cs, tot, -(ca * aYx))); break;
+    case 5: out = fmaf(-cs, tot, -(ca * aYy)); break;
+    case 6: out = -cs * tot; break;
+    default: out = delta * d * La; break;
   }
   return out;
 }
 
-// data_value written out: lane 0 the A-scan's structural term, lane 1 its
-// angiographic term, lanes 2..7 the six gradient components (3 V + c).
+// Output A-scan p = (i, j) by one warp: data_value written out.
 template <typename T>
-__device__ __forceinline__ void data_core(const DataArgs& A, int64_t p, int lane, const int base[6],
-                                          const float frac[6]) {
-  const float out = data_value<T>(A, p, lane, base, frac);
+__device__ __forceinline__ void data_ascan(const DataArgs& A, VolTab* tab, int64_t p, int i, int j, int lane) {
+  const float out = data_value<T>(A, tab, p, i, j, lane);
   const int64_t nasc = (int64_t)A.L.w * A.L.h;
-  if (lane == 0) A.str_out[p] = out;
-  else if (lane == 1) A.ang_out[p] = out;
-  else if (lane < 8 && A.grad) A.grad[(int64_t)(lane - 2) * nasc + p] = out;
-}
-
-// Output A-scan p by one warp from the volumes in global memory.
-template <typename T>
-__device__ __forceinline__ void data_ascan(const DataArgs& A, int64_t p, int lane) {
-  const LevelDev& L = A.L;
-  const int64_t nasc = (int64_t)L.w * L.h;
-  int base[6];
-  float frac[6];
-  split_displacement(A.disp, nasc, p, (int)(p % L.w), (int)(p / L.w), L, lane, base, frac);
-  data_core<T>(A, p, lane, base, frac);
+  const int v = lane >> 2;
+  if (lane & 3) return;
+  if (v == 0) A.str_out[p] = out;
+  else if (v == 7) A.ang_out[p] = out;
+  else if (A.grad) A.grad[(int64_t)(v - 1) * nasc + p] = out;
 }
 
 }  // namespace

@@ -10,19 +10,22 @@
 // over depth in the same pass.  The en-face angiography term (Eq. 6), the
 // resampled validity (Eq. 7) and delta (Eq. 8) are per-A-scan scalars.
 //
-// Mapping: one warp per output A-scan; a block's 8 warps take a tile of
-// 4 x 2 neighbouring A-scans (their 4 x 4 neighbourhoods overlap, which the
-// L1 cache turns into hits); 64 registers per thread, so 4 blocks (32 warps)
-// per SM keep loads in flight -- the kernel waits on memory latency more
-// than on arithmetic.  Depth is processed in blocks of 116
-// outputs; lane L (1..29) owns outputs kb + 4(L-1) .. +3.  Each lane loads
-// one aligned group of 4 input samples from each of the 16 transverse
-// neighbour columns with one 128-bit load per column (coalesced along depth
-// across the warp), forms the transverse interpolant T and its x/y
-// derivatives Tx, Ty for those 4 input depths, and gets the 3 neighbouring
-// input depths the 4-tap axial filter needs from the adjacent lanes by
-// shuffles.  Lanes 0, 30 and 31 only supply those halo values.  Per-A-scan
-// sums are reduced with a fixed butterfly, so results are deterministic.
+// Mapping: one warp per output A-scan; the sampling and its lane layout are
+// described in sample.cuh.  A block's 4 warps take a tile of 2 x 2
+// neighbouring A-scans (their 4 x 4 neighbourhoods overlap, which the L1 cache
+// turns into hits).  At 72 registers 7 blocks (28 warps) run per SM: the
+// kernel is bound by the L1 data pipe (volume loads, 5 wavefronts per 512
+// unaligned bytes; spilled registers cost it one more each) and by the
+// latency of its misses, so both fewer registers (more spills) and fewer
+// warps lose.  300 x 300 x 512, float32, data kernel alone: 64 registers
+// 517 us, 72 registers 488 us, 80 registers 500 us (529 us with depth-paired
+// multiply-adds and a per-lane prologue; bfloat16 535 -> 469 us; 64^3 19.2 ->
+// 16.6 us).
+//
+// The per-A-scan prologue (coordinate split, 24 weight pairs, 16 offsets) is
+// evaluated by a few lanes into a table in shared memory and the epilogue's 7
+// sums go through one reduce-scatter: at 64 samples of depth these were 1162
+// of a warp's 1958 instructions.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -34,19 +37,21 @@ namespace octmc {
 namespace {
 
 #ifndef OCTMC_DATA_MINB
-#define OCTMC_DATA_MINB 4
+#define OCTMC_DATA_MINB 7
 #endif
 #ifndef OCTMC_DTILE_X
-#define OCTMC_DTILE_X 4
+#define OCTMC_DTILE_X 2
 #endif
-constexpr int kDTileX = OCTMC_DTILE_X;  // direct kernel: a block's 8 A-scans as kDTileX x (8 / kDTileX)
+constexpr int kWarpsPerBlock = 4;
+constexpr int kDTileX = OCTMC_DTILE_X;  // a block's A-scans as kDTileX x (kWarpsPerBlock / kDTileX)
 constexpr int kDTileY = kWarpsPerBlock / kDTileX;
 
 // A-scan of warp `warp` of direct block b: tiles of kDTileX x kDTileY.
-__device__ __forceinline__ int64_t direct_ascan(const LevelDev& L, int b, int warp) {
-  const int tiles_x = (L.w + kDTileX - 1) / kDTileX;
-  const int i = (b % tiles_x) * kDTileX + warp % kDTileX, j = (b / tiles_x) * kDTileY + warp / kDTileX;
-  return (i < L.w && j < L.h) ? (int64_t)j * L.w + i : -1;
+__device__ __forceinline__ bool direct_ascan(const LevelDev& L, unsigned b, int warp, int* i, int* j) {
+  const unsigned tiles_x = (unsigned)(L.w + kDTileX - 1) / kDTileX;
+  *i = (int)(b % tiles_x) * kDTileX + warp % kDTileX;
+  *j = (int)(b / tiles_x) * kDTileY + warp / kDTileX;
+  return *i < L.w && *j < L.h;
 }
 
 __host__ __device__ inline int64_t direct_blocks(int w, int h) {
@@ -56,9 +61,11 @@ __host__ __device__ inline int64_t direct_blocks(int w, int h) {
 template <typename T>
 __global__ void __launch_bounds__(kWarpsPerBlock * kWarp, OCTMC_DATA_MINB)
 data_kernel(const DataArgs A) {
-  const int64_t p = direct_ascan(A.L, blockIdx.x, threadIdx.x >> 5);
-  if (p < 0) return;  // warp-uniform
-  data_ascan<T>(A, p, threadIdx.x & 31);
+  __shared__ VolTab tab[kWarpsPerBlock][2];
+  const int warp = threadIdx.x >> 5;
+  int i, j;
+  if (!direct_ascan(A.L, blockIdx.x, warp, &i, &j)) return;  // warp-uniform
+  data_ascan<T>(A, tab[warp], (int64_t)j * A.L.w + i, i, j, threadIdx.x & 31);
 }
 
 // Several problems ("slots") in one launch: grid (x, slots), block
@@ -71,9 +78,11 @@ __global__ void __launch_bounds__(kWarpsPerBlock * kWarp, OCTMC_DATA_MINB)
 data_multi_kernel(const __grid_constant__ DataMulti M) {
   const DataArgs& A = M.da[blockIdx.y];
   if ((int64_t)blockIdx.x >= direct_blocks(A.L.w, A.L.h)) return;
-  const int64_t p = direct_ascan(A.L, blockIdx.x, threadIdx.x >> 5);
-  if (p < 0) return;  // warp-uniform
-  data_ascan<T>(A, p, threadIdx.x & 31);
+  __shared__ VolTab tab[kWarpsPerBlock][2];
+  const int warp = threadIdx.x >> 5;
+  int i, j;
+  if (!direct_ascan(A.L, blockIdx.x, warp, &i, &j)) return;  // warp-uniform
+  data_ascan<T>(A, tab[warp], (int64_t)j * A.L.w + i, i, j, threadIdx.x & 31);
 }
 
 }  // namespace

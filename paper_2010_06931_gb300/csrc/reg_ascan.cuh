@@ -24,21 +24,19 @@ __device__ __forceinline__ float huber_r(float x, float inv_eps, float* dl) {
 // gradient and the float64 gradient of component 3 V + c = lane; partial
 // sums into acc (S^str, S^ang, R, grad . dir) and the running max |grad|.
 template <typename T>
-__device__ __forceinline__ void eval_ascan(const DataArgs& D, double* __restrict__ grad, const double* __restrict__ dir,
+__device__ __forceinline__ void eval_ascan(const DataArgs& D, VolTab* tab, double* __restrict__ grad, const double* __restrict__ dir,
                                            int64_t p, int lane, float two_mu_s, float inv_eps_r, float alpha_d,
                                            double* acc, unsigned long long* gmx) {
   const LevelDev& L = D.L;
   const int64_t plane = (int64_t)L.w * L.h;
   const double* xt = D.disp;
-  int base[6];
-  float frac[6];
-  split_displacement(xt, plane, p, (int)(p % L.w), (int)(p / L.w), L, lane, base, frac);
-  const float out = data_value<T>(D, p, lane, base, frac);
-  // lane 0: the A-scan's structural term, lane 1 its angiographic term,
-  // lane 2 + q: the data-term gradient of component q
-  const float gdat = __shfl_sync(0xffffffffu, out, (lane + 2) & 31);
+  const float out = data_value<T>(D, tab, p, (int)(p % L.w), (int)(p / L.w), lane);
+  // lane 0: the A-scan's structural term, lane 28 its angiographic term,
+  // lane 4 (1 + q): the data-term gradient of component q
+  const float gdat = __shfl_sync(0xffffffffu, out, (4 * (lane + 1)) & 31);
+  const float ang = __shfl_sync(0xffffffffu, out, 28);
   if (lane == 0) acc[0] += widen_exact(out);
-  if (lane == 1) acc[1] += widen_exact(out);
+  if (lane == 1) acc[1] += widen_exact(ang);
   if (lane < 6) {
     const int V_ = lane / 3, c_ = lane % 3;
     const int nx = L.next[V_][p], pv = L.prev[V_][p];

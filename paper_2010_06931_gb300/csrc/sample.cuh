@@ -1,8 +1,7 @@
-// Displaced Catmull-Rom sampling of one A-scan by one warp, shared by the
-// data-term kernel and the final resampling (Ploner et al., Eq. 2 and
-// Sec. 2.1): coordinate split, per-volume setup, the lane-parallel
-// transverse 4x4 interpolation of aligned groups of 4 input samples and the
-// 4-tap axial filter with its halo shuffles.
+// Displaced Catmull-Rom sampling of one A-scan by one warp, with its
+// derivatives (Ploner et al., Eq. 2): coordinate split and interpolation
+// tables, the lane-parallel transverse 4x4 interpolation of aligned groups of
+// 4 input samples and the 4-tap axial filter with its halo shuffles.
 //
 // Depth is processed in blocks of 116 outputs; lane L (1..29) owns outputs
 // kb + 4(L-1) .. +3, loads one aligned group of 4 input samples from each of
@@ -10,71 +9,110 @@
 // (coalesced along depth across the warp), and gets the neighbouring input
 // depths the axial filter needs from the adjacent lanes by shuffles.  Lanes
 // 0, 30 and 31 only supply those halo values.
+//
+// The packed multiply-add (fma.rn.f32x2: two lanes, one issue slot, two FMA
+// pipe cycles) takes a scalar broadcast to both halves at no cost but needs
+// its pairs in aligned registers.  So the pairs here are (value, derivative):
+// the weights come as pairs, each sample is broadcast, and the results of one
+// stage are the pairs of the next; pairing neighbouring depths instead costs
+// moves in the axial filter, whose taps start at odd offsets (462.4 M against
+// 370.3 M warp instructions per launch at 300 x 300 x 512 with the rest of
+// the kernel as it is now).
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+#include <stddef.h>
 
 #include "common.cuh"
 
 namespace octmc {
 namespace {
 
-constexpr int kWarpsPerBlock = 8;
 constexpr int kOutLanes = 29;
 constexpr int kOutPerIter = 4 * kOutLanes;
 constexpr unsigned kFull = 0xffffffffu;
 
-struct Vol {
-  const void* base;    // the volume; addressed in groups of 4 samples
-  unsigned roff[4];    // row offsets (in groups) of the 4 neighbour rows
-  unsigned coff[4];    // column offsets (in groups) of the 4 neighbour columns
-  float wx[4], dwx[4], wy[4], dwy[4], wz[4], dwz[4];
-  int q, r;            // floor(dz) = 4 q + r, 0 <= r < 4
-  int bx, by;          // floor of the transverse coordinates
+// Sampling of one volume at one A-scan: the offsets of the 4 x 4 neighbour
+// columns and the interpolation weights, in shared memory (one table per warp
+// and volume; every lane reads the same address).
+struct alignas(16) VolTab {
+  float2 wx[4];     // x weights as (derivative, value)
+  float2 wz[4];     // z weights as (value, derivative)
+  float2 wy[4];     // y weights as (value, derivative)
+  unsigned off[8];  // offsets (in groups of 4 samples) of the 4 neighbour rows, then columns
 };
 
-// Coordinate split of the 6 displacement values of A-scan (i, j) by lanes
-// 0..5 (lane = 3 V + c), broadcast to the warp: floor(u) and the float
-// fraction for u = i + dx and u = j + dy clamped to [-4, n + 3] (beyond that
-// every tap is an edge sample) and u = dz clamped to +-(d + 8) (all depth
-// taps are then edge samples).  Integer arithmetic only (split_exact).
-__device__ __forceinline__ void split_displacement(const double* disp, int64_t nasc, int64_t p, int i,
-                                                   int j, const LevelDev& L, int lane, int base[6],
-                                                   float frac[6]) {
-  int b = 0;
-  float t = 0.f;
-  if (lane < 6) {
-    const int c = lane % 3;
-    const unsigned long long bits =
-        (unsigned long long)__double_as_longlong(disp[(int64_t)lane * nasc + p]);
-    if (c == 0) split_exact(bits, i, -4, L.w + 3, &b, &t);
-    else if (c == 1) split_exact(bits, j, -4, L.h + 3, &b, &t);
-    else split_exact(bits, 0, -L.d - 8, L.d + 8, &b, &t);
-  }
-#pragma unroll
-  for (int c = 0; c < 6; c++) {
-    base[c] = __shfl_sync(0xffffffffu, b, c);
-    frac[c] = __shfl_sync(0xffffffffu, t, c);
-  }
+struct Vol {
+  const void* base;    // the volume; addressed in groups of 4 samples
+  unsigned tab;        // shared-memory address of its VolTab
+  int q, r;            // floor(dz) = 4 q + r, 0 <= r < 4
+  int bx, by;          // floor of the transverse coordinates
+  float ts;            // the fraction along the scan's slow axis (y for X, x for Y), Eq. 7
+};
+
+// Table reads.  Volatile: each is one broadcast load at the place of use, so
+// the table is not kept in (or spilled from) the registers of the depth loop.
+__device__ __forceinline__ void lds4(unsigned addr, float2& a, float2& b) {
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a.x), "=f"(a.y), "=f"(b.x), "=f"(b.y) : "r"(addr));
+}
+__device__ __forceinline__ void lds2(unsigned addr, float2& a) {
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(a.x), "=f"(a.y) : "r"(addr));
+}
+__device__ __forceinline__ void lds4u(unsigned addr, unsigned u[4]) {
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]) : "r"(addr));
 }
 
-__device__ __forceinline__ void setup_vol(Vol& V, const void* vol, const LevelDev& L, const int base[3],
-                                          const float frac[3]) {
-  V.bx = base[0];
-  V.by = base[1];
-  const int kz0 = base[2];
-  V.q = kz0 >> 2;  // arithmetic shift: floor division by 4
-  V.r = kz0 & 3;
-  keys_weights(frac[0], V.wx, V.dwx);
-  keys_weights(frac[1], V.wy, V.dwy);
-  keys_weights(frac[2], V.wz, V.dwz);
-  const unsigned nq = (unsigned)(L.dp >> 2);
+// Coordinate split of the 6 displacement values of A-scan (i, j) by lanes
+// 0..5 (lane = 3 V + c): floor(u) and the float fraction for u = i + dx and
+// u = j + dy clamped to [-4, n + 3] (beyond that every tap is an edge sample)
+// and u = dz clamped to +-(d + 8) (all depth taps are then edge samples).
+// Integer arithmetic only (split_exact).  The lane then evaluates the 4
+// weights of its component, and lanes 0..15 the neighbour offsets, once per
+// A-scan; the warp reads them back from shared memory.
+__device__ __forceinline__ void setup_pair(Vol& VX, Vol& VY, VolTab* tab, const double* disp, int64_t nasc, int64_t p,
+                                           int i, int j, const LevelDev& L, int lane) {
+  int b = 0;
+  float t = 0.f;
+  const int c = lane < 3 ? lane : lane - 3;
+  if (lane < 6) {
+    const unsigned long long bits =
+        (unsigned long long)__double_as_longlong(disp[(int64_t)lane * nasc + p]);
+    const int off = c == 0 ? i : (c == 1 ? j : 0);
+    const int lo = c == 2 ? -L.d - 8 : -4;
+    const int hi = c == 0 ? L.w + 3 : (c == 1 ? L.h + 3 : L.d + 8);
+    split_exact(bits, off, lo, hi, &b, &t);
+    float w[4], dw[4];
+    keys_weights(t, w, dw);
+    VolTab& W = tab[lane < 3 ? 0 : 1];
+    float2* dst = c == 0 ? W.wx : (c == 1 ? W.wy : W.wz);
 #pragma unroll
-  for (int a = 0; a < 4; a++) {
-    V.roff[a] = (unsigned)clampi(V.by - 1 + a, L.h) * (unsigned)L.w * nq;
-    V.coff[a] = (unsigned)clampi(V.bx - 1 + a, L.w) * nq;
+    for (int a = 0; a < 4; a++) dst[a] = c == 0 ? make_float2(dw[a], w[a]) : make_float2(w[a], dw[a]);
   }
-  V.base = vol;
+  VX.bx = __shfl_sync(kFull, b, 0);
+  VX.by = __shfl_sync(kFull, b, 1);
+  const int zx = __shfl_sync(kFull, b, 2);
+  VY.bx = __shfl_sync(kFull, b, 3);
+  VY.by = __shfl_sync(kFull, b, 4);
+  const int zy = __shfl_sync(kFull, b, 5);
+  VX.ts = __shfl_sync(kFull, t, 1);
+  VY.ts = __shfl_sync(kFull, t, 3);
+  VX.q = zx >> 2;  // arithmetic shift: floor division by 4
+  VX.r = zx & 3;
+  VY.q = zy >> 2;
+  VY.r = zy & 3;
+  if (lane < 16) {  // lanes 0..7: volume X, 8..15: volume Y; 4 rows, then 4 columns
+    const unsigned nq = (unsigned)(L.dp >> 2);
+    const int a = lane & 3;
+    const bool isY = lane >= 8;
+    const unsigned off = (lane & 4) ? (unsigned)clampi((isY ? VY.bx : VX.bx) - 1 + a, L.w) * nq
+                                    : (unsigned)clampi((isY ? VY.by : VX.by) - 1 + a, L.h) * (unsigned)L.w * nq;
+    tab[isY ? 1 : 0].off[lane & 7] = off;
+  }
+  __syncwarp();
+  VX.tab = (unsigned)__cvta_generic_to_shared(tab);
+  VY.tab = VX.tab + (unsigned)sizeof(VolTab);
+  VX.base = L.sx;
+  VY.base = L.sy;
 }
 
 // Four consecutive samples (one aligned group) widened to float: float32
@@ -113,156 +151,112 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   return d;
 }
 
-// Four consecutive depth samples as two packed pairs (k, k+1), (k+2, k+3).
-struct Q4 {
-  float2 lo, hi;
-};
-
-__device__ __forceinline__ Q4 q4(const float4& v) { return {make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
-__device__ __forceinline__ Q4 q4zero() { return {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-
-// acc += w * s on all four samples (w broadcast to both halves)
-__device__ __forceinline__ void qfma(Q4& acc, float2 w, const Q4& s) {
-  acc.lo = ffma2(w, s.lo, acc.lo);
-  acc.hi = ffma2(w, s.hi, acc.hi);
+__device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
 }
+__device__ __forceinline__ float2 both(float s) { return make_float2(s, s); }
 
-__device__ __forceinline__ float4 f4(const Q4& q) { return make_float4(q.lo.x, q.lo.y, q.hi.x, q.hi.y); }
-
-__device__ __forceinline__ void fma4(float4& acc, float w, const float4& s) {
-  acc.x = fmaf(w, s.x, acc.x);
-  acc.y = fmaf(w, s.y, acc.y);
-  acc.z = fmaf(w, s.z, acc.z);
-  acc.w = fmaf(w, s.w, acc.w);
-}
-
-__device__ __forceinline__ float4 bcast(float v) { return make_float4(v, v, v, v); }
-
-// Axial 4-tap filter for the lane's 4 outputs.  e[1..4] hold the lane's
-// own input group, e[0] the last sample of lane-1's group, e[5..8] lane+1's
-// group and e[9] the first sample of lane+2's.  Output o, tap c reads
-// e[R + o + c], where R = floor(dz) mod 4.
+// Axial 4-tap filter of NQ quantities for the lane's 4 outputs: the lane's
+// group of each is e[1..4], e[0] the last sample of lane - 1's group, e[5..8]
+// lane + 1's group and e[9] the first sample of lane + 2's.  Output o, tap c
+// reads e[R + o + c], where R = floor(dz) mod 4.
 template <int R>
-__device__ __forceinline__ void axial(const float4& T, const float4& Tx, const float4& Ty,
-                                      const float wz[4], const float dwz[4], float I[4], float Iz[4],
-                                      float Ix[4], float Iy[4]) {
+__device__ __forceinline__ void halo(float e[10]) {
+  if (R == 0) e[0] = __shfl_up_sync(kFull, e[4], 1);
+  e[5] = __shfl_down_sync(kFull, e[1], 1);
+  e[6] = __shfl_down_sync(kFull, e[2], 1);
+  if (R >= 1) e[7] = __shfl_down_sync(kFull, e[3], 1);
+  if (R >= 2) e[8] = __shfl_down_sync(kFull, e[4], 1);
+  if (R == 3) e[9] = __shfl_down_sync(kFull, e[1], 2);
+}
+
+template <int R>
+__device__ __forceinline__ void axial(const float T[4], const float2 Txy[4], const float2 wz[4], float2 Iz[4],
+                                      float2 Ixy[4]) {
   float e[10], ex[10], ey[10];
-  e[1] = T.x; e[2] = T.y; e[3] = T.z; e[4] = T.w;
-  ex[1] = Tx.x; ex[2] = Tx.y; ex[3] = Tx.z; ex[4] = Tx.w;
-  ey[1] = Ty.x; ey[2] = Ty.y; ey[3] = Ty.z; ey[4] = Ty.w;
-  if (R == 0) {
-    e[0] = __shfl_up_sync(kFull, T.w, 1);
-    ex[0] = __shfl_up_sync(kFull, Tx.w, 1);
-    ey[0] = __shfl_up_sync(kFull, Ty.w, 1);
-  }
-  e[5] = __shfl_down_sync(kFull, T.x, 1);
-  ex[5] = __shfl_down_sync(kFull, Tx.x, 1);
-  ey[5] = __shfl_down_sync(kFull, Ty.x, 1);
-  e[6] = __shfl_down_sync(kFull, T.y, 1);
-  ex[6] = __shfl_down_sync(kFull, Tx.y, 1);
-  ey[6] = __shfl_down_sync(kFull, Ty.y, 1);
-  if (R >= 1) {
-    e[7] = __shfl_down_sync(kFull, T.z, 1);
-    ex[7] = __shfl_down_sync(kFull, Tx.z, 1);
-    ey[7] = __shfl_down_sync(kFull, Ty.z, 1);
-  }
-  if (R >= 2) {
-    e[8] = __shfl_down_sync(kFull, T.w, 1);
-    ex[8] = __shfl_down_sync(kFull, Tx.w, 1);
-    ey[8] = __shfl_down_sync(kFull, Ty.w, 1);
-  }
-  if (R == 3) {
-    e[9] = __shfl_down_sync(kFull, T.x, 2);
-    ex[9] = __shfl_down_sync(kFull, Tx.x, 2);
-    ey[9] = __shfl_down_sync(kFull, Ty.x, 2);
-  }
-#ifndef OCTMC_AXIAL_PACKED
-#define OCTMC_AXIAL_PACKED 1
-#endif
-#if OCTMC_AXIAL_PACKED
-  // outputs in packed pairs (o, o + 1); each half adds its 4 taps in the
-  // scalar order
 #pragma unroll
-  for (int o = 0; o < 4; o += 2) {
-    float2 a = make_float2(0.f, 0.f), az = a, ax = a, ay = a;
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      const float2 w = make_float2(wz[c], wz[c]), dw = make_float2(dwz[c], dwz[c]);
-      const float2 ev = make_float2(e[R + o + c], e[R + o + 1 + c]);
-      a = ffma2(w, ev, a);
-      az = ffma2(dw, ev, az);
-      ax = ffma2(w, make_float2(ex[R + o + c], ex[R + o + 1 + c]), ax);
-      ay = ffma2(w, make_float2(ey[R + o + c], ey[R + o + 1 + c]), ay);
-    }
-    I[o] = a.x; I[o + 1] = a.y;
-    Iz[o] = az.x; Iz[o + 1] = az.y;
-    Ix[o] = ax.x; Ix[o + 1] = ax.y;
-    Iy[o] = ay.x; Iy[o + 1] = ay.y;
+  for (int k = 0; k < 4; k++) {
+    e[1 + k] = T[k];
+    ex[1 + k] = Txy[k].x;
+    ey[1 + k] = Txy[k].y;
   }
-#else
+  halo<R>(e);
+  halo<R>(ex);
+  halo<R>(ey);
 #pragma unroll
   for (int o = 0; o < 4; o++) {
-    float a = 0.f, az = 0.f, ax = 0.f, ay = 0.f;
+    float2 a = fmul2(wz[0], both(e[R + o]));
+    float2 g = fmul2(both(wz[0].x), make_float2(ex[R + o], ey[R + o]));
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-      a = fmaf(wz[c], e[R + o + c], a);
-      az = fmaf(dwz[c], e[R + o + c], az);
-      ax = fmaf(wz[c], ex[R + o + c], ax);
-      ay = fmaf(wz[c], ey[R + o + c], ay);
+    for (int c = 1; c < 4; c++) {
+      a = ffma2(wz[c], both(e[R + o + c]), a);
+      g = ffma2(both(wz[c].x), make_float2(ex[R + o + c], ey[R + o + c]), g);
     }
-    I[o] = a; Iz[o] = az; Ix[o] = ax; Iy[o] = ay;
+    Iz[o] = a;
+    Ixy[o] = g;
   }
-#endif
 }
 
-// Interpolated values (and their displacement derivatives) of one volume
-// at the lane's 4 outputs.  qk: first input depth of the lane's group
-// (samples, may lie outside the volume); qc: index of that group's (clamped)
-// samples in the volume.
+// (I, dI/dz) and (dI/dx, dI/dy) of one volume at the lane's 4 outputs.  qk:
+// first input depth of the lane's group (samples, may lie outside the
+// volume); qc: index of that group's (clamped) samples in the volume.
 template <typename S>
-__device__ __forceinline__ void sample_group(const Vol& V, int qk, unsigned qc, int dp, float I[4], float Iz[4],
-                                             float Ix[4], float Iy[4]) {
-  // transverse 4 x 4 interpolation of the group and its x / y derivatives,
-  // in packed pairs along depth (same operations and order as scalar FMAs)
-  Q4 Tq = q4zero(), Txq = q4zero(), Tyq = q4zero();
+__device__ __forceinline__ void sample_group(const Vol& V, int qk, unsigned qc, int dp, float2 Iz[4], float2 Ixy[4]) {
+  float T[4];
+  float2 Txy[4], wx[4], wz[4];
+  unsigned coff[4], roff[4];
+  lds4u(V.tab + offsetof(VolTab, off) + 16, coff);
+  lds4u(V.tab + offsetof(VolTab, off), roff);
+  lds4(V.tab + offsetof(VolTab, wx), wx[0], wx[1]);
+  lds4(V.tab + offsetof(VolTab, wx) + 16, wx[2], wx[3]);
 #pragma unroll
   for (int b = 0; b < 4; b++) {
-    Q4 U = q4zero(), Ux = q4zero();
+    float2 U[4];  // (d/dx, value) of row b
+    float2 wy;
+    lds2(V.tab + offsetof(VolTab, wy) + 8 * b, wy);
 #pragma unroll
     for (int a = 0; a < 4; a++) {
-      const unsigned idx = V.roff[b] + V.coff[a] + qc;
-      const Q4 s = q4(load4<S>(V.base, idx));
-      qfma(U, make_float2(V.wx[a], V.wx[a]), s);
-      qfma(Ux, make_float2(V.dwx[a], V.dwx[a]), s);
+      const float4 f = load4<S>(V.base, roff[b] + coff[a] + qc);
+      const float s[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+      for (int k = 0; k < 4; k++) U[k] = a == 0 ? fmul2(wx[0], both(s[k])) : ffma2(wx[a], both(s[k]), U[k]);
     }
-    qfma(Tq, make_float2(V.wy[b], V.wy[b]), U);
-    qfma(Txq, make_float2(V.wy[b], V.wy[b]), Ux);
-    qfma(Tyq, make_float2(V.dwy[b], V.dwy[b]), U);
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      Txy[k] = b == 0 ? fmul2(wy, U[k]) : ffma2(wy, U[k], Txy[k]);
+      T[k] = b == 0 ? wy.x * U[k].y : fmaf(wy.x, U[k].y, T[k]);
+    }
   }
-  float4 T = f4(Tq), Tx = f4(Txq), Ty = f4(Tyq);
   // groups entirely before sample 0 / after the last sample hold the edge value
   if (qk < 0) {
-    T = bcast(T.x); Tx = bcast(Tx.x); Ty = bcast(Ty.x);
+#pragma unroll
+    for (int k = 1; k < 4; k++) { T[k] = T[0]; Txy[k] = Txy[0]; }
   } else if (qk >= dp) {
-    T = bcast(T.w); Tx = bcast(Tx.w); Ty = bcast(Ty.w);
+#pragma unroll
+    for (int k = 0; k < 3; k++) { T[k] = T[3]; Txy[k] = Txy[3]; }
   }
+  lds4(V.tab + offsetof(VolTab, wz), wz[0], wz[1]);
+  lds4(V.tab + offsetof(VolTab, wz) + 16, wz[2], wz[3]);
   switch (V.r) {
-    case 0: axial<0>(T, Tx, Ty, V.wz, V.dwz, I, Iz, Ix, Iy); break;
-    case 1: axial<1>(T, Tx, Ty, V.wz, V.dwz, I, Iz, Ix, Iy); break;
-    case 2: axial<2>(T, Tx, Ty, V.wz, V.dwz, I, Iz, Ix, Iy); break;
-    default: axial<3>(T, Tx, Ty, V.wz, V.dwz, I, Iz, Ix, Iy); break;
+    case 0: axial<0>(T, Txy, wz, Iz, Ixy); break;
+    case 1: axial<1>(T, Txy, wz, Iz, Ixy); break;
+    case 2: axial<2>(T, Txy, wz, Iz, Ixy); break;
+    default: axial<3>(T, Txy, wz, Iz, Ixy); break;
   }
 }
 
-// Interpolated values (and their displacement derivatives) of one volume
-// at the lane's 4 outputs of the depth block starting at kb, from the
-// volume in global memory.
+// The same at the lane's 4 outputs of the depth block starting at kb.
 template <typename S>
-__device__ __forceinline__ void sample_block(const Vol& V, int kb, int lane, int dp, float I[4],
-                                             float Iz[4], float Ix[4], float Iy[4]) {
+__device__ __forceinline__ void sample_block(const Vol& V, int kb, int lane, int dp, float2 Iz[4], float2 Ixy[4]) {
   const int qk = kb + 4 * V.q + 4 * (lane - 1);  // first input depth of the lane's group
   const unsigned qc = (unsigned)(min(max(qk, 0), dp - 4) >> 2);
-  sample_group<S>(V, qk, qc, dp, I, Iz, Ix, Iy);
+  sample_group<S>(V, qk, qc, dp, Iz, Ixy);
 }
 
 }  // namespace
