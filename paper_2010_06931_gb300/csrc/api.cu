@@ -644,6 +644,7 @@ void eval_batch(cudaStream_t st, const std::vector<EvalReq>& reqs) {
       R.counter = P->counters + 1;
       R.ctl = nullptr;
       R.h_branch = 0;
+      R.axial = false;
       RM.b0[k + 1] = RM.b0[k] + reg_grid_blocks(n);
     }
     // The mean-term sums only feed the regulariser kernel: they run on a side
@@ -1021,14 +1022,58 @@ void ensure_prealign(octmc_problem* P) {
   CK(cudaMallocHost(&P->pre_aux_host, 2 * sizeof(double)));
 }
 
+// Enqueues the structural objective (delta_0 = 0, eta = 1) of a field without
+// transverse displacement, and its axial gradient components; the result is
+// copied to P->res_host.  The transverse planes of D and G are neither read
+// nor written.
+void eval_axial(octmc_problem* P, int l, const double* D, double* G) {
+  const Level& Lv = P->lv[l];
+  DataArgs A;
+  std::memset(&A, 0, sizeof(A));
+  A.L = Lv.dev;
+  A.disp = D;
+  A.str_out = P->str;
+  A.ang_out = P->ang;
+  A.grad = G ? P->gdata : nullptr;
+  A.eta = 1.0;
+  A.eps_h = (float)P->desc.eps_h;
+  A.loss = P->desc.loss;
+  RegArgs R;
+  std::memset(&R, 0, sizeof(R));
+  R.L = Lv.dev;
+  R.disp = D;
+  R.grad = G;
+  R.gdata = P->gdata;
+  R.str_in = P->str;
+  R.ang_in = P->ang;
+  R.alpha = P->desc.alpha;
+  R.eps_r = P->desc.eps_r;
+  R.mu = Lv.mu;
+  R.eta = 1.0;
+  R.axial = true;
+  R.result = P->res;
+  R.partials = P->partials;
+  R.counter = P->counters + 1;
+  const bool prof = P->profile;
+  CK(launch_msum(D, P->plane(l), P->res, P->partials, P->counters + 0, P->st, true));
+  if (prof) CK(cudaEventRecord(P->ev0, P->st));
+  CK(launch_data_column(A, P->st));
+  if (prof) {
+    CK(cudaEventRecord(P->ev1, P->st));
+    P->prof_pending = true;
+  }
+  CK(launch_reg(R, P->st));
+  CK(cudaMemcpyAsync(P->res_host, P->res, sizeof(EvalResult), cudaMemcpyDeviceToHost, P->st));
+}
+
 // f (host) and, if gprm, the parameter gradient (device); with dir also
 // gprm . dir in *gdir.
 void prealign_eval_impl(octmc_problem* P, int l, const double* prm, double* gprm, const double* dir, double* f,
                         double* gdir) {
   ensure_prealign(P);
   const LevelDev& L = P->lv[l].dev;
-  CK(launch_prm_to_disp(prm, L.w, L.h, P->pre_D, P->st));
-  eval_batch(P->st, {EvalReq{P, l, P->pre_D, gprm ? P->pre_G : nullptr, nullptr, 1.0, 0.0}});
+  CK(launch_prm_to_disp(prm, L.w, L.h, P->pre_D, false, P->st));
+  eval_axial(P, l, P->pre_D, gprm ? P->pre_G : nullptr);
   if (gprm) {
     CK(launch_grad_to_prm(P->pre_G, L.w, L.h, prm, gprm, P->pre_aux, P->st));
     if (dir) CK(launch_prm_dot(gprm, dir, prealign_n(P, l), P->pre_aux + 1, P->st));
@@ -1491,7 +1536,7 @@ int octmc_prealign_disp(octmc_problem* p, int level, const double* prm, double* 
   if (!valid_level(p, level) || !prm || !disp) return OCTMC_ERR_INVALID_ARG;
   return guarded([&] {
     const LevelDev& L = p->lv[level].dev;
-    CK(launch_prm_to_disp(prm, L.w, L.h, disp, p->st));
+    CK(launch_prm_to_disp(prm, L.w, L.h, disp, true, p->st));
     CK(cudaStreamSynchronize(p->st));
     return OCTMC_OK;
   });
@@ -1538,7 +1583,7 @@ int octmc_prealign_full(octmc_problem* p, double* prm_out, double* disp0_out, oc
     }
     if (disp0_out) {
       const LevelDev& F = p->lv[0].dev;
-      CK(launch_prm_to_disp(cur, F.w, F.h, disp0_out, p->st));
+      CK(launch_prm_to_disp(cur, F.w, F.h, disp0_out, true, p->st));
       CK(cudaStreamSynchronize(p->st));
     }
     return rc;

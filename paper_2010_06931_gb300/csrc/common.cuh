@@ -272,6 +272,7 @@ struct RegArgs {
   const float* ang_in;    // [h*w]
   double alpha, eps_r, mu, eta;
   const double* eta_dev;  // if not null: eta is read here
+  bool axial;             // only the axial components (the transverse ones of disp are 0)
   EvalResult* result;     // device
   double* partials;       // [grid][8] scratch
   unsigned* counter;      // zero-initialised, reset by the last block
@@ -317,14 +318,18 @@ cudaError_t launch_data_multi(const DataMulti& M, int dtype, cudaStream_t s);
 cudaError_t launch_msum_multi(const MsumMulti& M, cudaStream_t s);
 cudaError_t launch_reg_multi(const RegMulti& M, cudaStream_t s);
 cudaError_t launch_data(const DataArgs& a, cudaStream_t s);
+// the field has no transverse displacement: axial gradient components only
+cudaError_t launch_data_column(const DataArgs& a, cudaStream_t s);
+// axial: only the axial component's sum (the others are set to 0)
 cudaError_t launch_msum(const double* disp, int64_t plane, EvalResult* res, double* partials,
-                        unsigned* counter, cudaStream_t s);
+                        unsigned* counter, cudaStream_t s, bool axial = false);
 cudaError_t launch_reg(const RegArgs& a, cudaStream_t s);
 int reg_grid_blocks(int64_t n_ascans);
 int msum_grid_blocks();
 
 // Rough axial prealignment (stage 1 of Sec. 2.1).
-cudaError_t launch_prm_to_disp(const double* prm, int w, int h, double* disp, cudaStream_t s);
+// all: all six planes, else only the two axial ones
+cudaError_t launch_prm_to_disp(const double* prm, int w, int h, double* disp, bool all, cudaStream_t s);
 cudaError_t launch_grad_to_prm(const double* g, int w, int h, const double* prm, double* gprm, double* T_out,
                                cudaStream_t s);
 cudaError_t launch_prm_dot(const double* a, const double* b, int n, double* out, cudaStream_t s);

@@ -160,6 +160,118 @@ __device__ __forceinline__ float data_value(const DataArgs& A, VolTab* tab, int6
   return out;
 }
 
+// ---- fields without transverse displacement (the axial prealignment)
+// At dx = dy = 0 the transverse weights are exactly (0, 1, 0, 0), so the
+// interpolant is the A-scan's own column filtered along depth: one column per
+// scan instead of 16, the same floats in the same order as data_value.  Only
+// the axial gradient components (c = 2) are formed.
+template <int R>
+__device__ __forceinline__ void axial_z(const float T[4], const float2 wz[4], float2 Iz[4]) {
+  float e[10];
+#pragma unroll
+  for (int k = 0; k < 4; k++) e[1 + k] = T[k];
+  halo<R>(e);
+#pragma unroll
+  for (int o = 0; o < 4; o++) {
+    float2 a = fmul2(wz[0], both(e[R + o]));
+#pragma unroll
+    for (int c = 1; c < 4; c++) a = ffma2(wz[c], both(e[R + o + c]), a);
+    Iz[o] = a;
+  }
+}
+
+__device__ __forceinline__ void column_filter(float4 f, int qk, int dp, int r, const float2 wz[4], float2 Iz[4]) {
+  // groups entirely before sample 0 / after the last sample hold the edge value
+  if (qk < 0) f.y = f.z = f.w = f.x;
+  else if (qk >= dp) f.x = f.y = f.z = f.w;
+  const float T[4] = {f.x, f.y, f.z, f.w};
+  switch (r) {
+    case 0: axial_z<0>(T, wz, Iz); break;
+    case 1: axial_z<1>(T, wz, Iz); break;
+    case 2: axial_z<2>(T, wz, Iz); break;
+    default: axial_z<3>(T, wz, Iz); break;
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void data_column(const DataArgs& A, int64_t p, int i, int j, int lane) {
+  const LevelDev& L = A.L;
+  const int64_t nasc = (int64_t)L.w * L.h;
+  int b = 0;
+  float t = 0.f;
+  if (lane < 2)  // lane = scan
+    split_exact((unsigned long long)__double_as_longlong(A.disp[(int64_t)(3 * lane + 2) * nasc + p]), 0, -L.d - 8,
+                L.d + 8, &b, &t);
+  const int zx = __shfl_sync(kFull, b, 0), zy = __shfl_sync(kFull, b, 1);
+  float2 wx[4], wy[4];  // axial weights of scan X, scan Y
+  {
+    float w[4], dw[4];
+    keys_weights(__shfl_sync(kFull, t, 0), w, dw);
+#pragma unroll
+    for (int a = 0; a < 4; a++) wx[a] = make_float2(w[a], dw[a]);
+    keys_weights(__shfl_sync(kFull, t, 1), w, dw);
+#pragma unroll
+    for (int a = 0; a < 4; a++) wy[a] = make_float2(w[a], dw[a]);
+  }
+  const unsigned col = (unsigned)p * (unsigned)(L.dp >> 2);
+  const float inv_eps = 1.0f / A.eps_h;
+  const bool ssd = (A.loss == OCTMC_LOSS_SSD);
+  int left = (lane >= 1 && lane <= kOutLanes) ? L.d - 4 * (lane - 1) : 0;
+  // first input depth of the lane's group, as in sample_block
+  int qx = 4 * (zx >> 2) + 4 * (lane - 1), qy = 4 * (zy >> 2) + 4 * (lane - 1);
+  auto load = [&](const void* vol, int qk) { return load4<T>(vol, col + (unsigned)(min(max(qk, 0), L.dp - 4) >> 2)); };
+  float4 fx = load(L.sx, qx), fy = load(L.sy, qy);
+  float Ls = 0.f, gx = 0.f, gy = 0.f;
+  for (int kb = 0; kb < L.d; kb += kOutPerIter, left -= kOutPerIter) {
+    // the next depth block's loads are in flight while this one is computed
+    float4 nx, ny;
+    const bool more = kb + kOutPerIter < L.d;
+    if (more) {
+      nx = load(L.sx, qx + kOutPerIter);
+      ny = load(L.sy, qy + kOutPerIter);
+    }
+    float2 X[4], Y[4];
+    column_filter(fx, qx, L.dp, zx & 3, wx, X);
+    column_filter(fy, qy, L.dp, zy & 3, wy, Y);
+    auto add = [&](int o) {
+      float Lv, dL;
+      loss_grad(X[o].x - Y[o].x, inv_eps, ssd, &Lv, &dL);
+      Ls += Lv;
+      gx = fmaf(dL, X[o].y, gx);
+      gy = fmaf(dL, Y[o].y, gy);
+    };
+    if (left >= 4) {
+#pragma unroll
+      for (int o = 0; o < 4; o++) add(o);
+    } else if (left > 0) {
+      add(0);
+      if (left > 1) add(1);
+      if (left > 2) add(2);
+    }
+    if (more) {
+      fx = nx;
+      fy = ny;
+    }
+    qx += kOutPerIter;
+    qy += kOutPerIter;
+  }
+  Ls = warp_sum(Ls);
+  gx = warp_sum(gx);
+  gy = warp_sum(gy);
+  if (lane > 2) return;
+  // validity and angiography at the A-scan itself (Eq. 6-8)
+  float delta = (float)A.delta0;
+  if (L.vx) delta *= L.vx[j];
+  if (L.vy) delta *= L.vy[i];
+  float La = 0.f, dLa = 0.f;
+  if (L.ax) loss_grad(L.ax[p] - L.ay[p], inv_eps, ssd, &La, &dLa);
+  const float eta = (float)(A.eta_dev ? *A.eta_dev : A.eta);
+  const float cs = eta * (1.0f - delta);
+  if (lane == 0) A.str_out[p] = (1.0f - delta) * Ls;
+  else if (lane == 1) A.ang_out[p] = delta * (float)L.d * La;
+  if (A.grad && lane >= 1) A.grad[(lane == 1 ? 2 : 5) * nasc + p] = lane == 1 ? cs * gx : -cs * gy;
+}
+
 // Output A-scan p = (i, j) by one warp: data_value written out.
 template <typename T>
 __device__ __forceinline__ void data_ascan(const DataArgs& A, VolTab* tab, int64_t p, int i, int j, int lane) {

@@ -85,6 +85,18 @@ data_multi_kernel(const __grid_constant__ DataMulti M) {
   data_ascan<T>(A, tab[warp], (int64_t)j * A.L.w + i, i, j, threadIdx.x & 31);
 }
 
+// The data term of a field without transverse displacement: one warp per
+// A-scan, two columns read once.  Bound by HBM; 8-warp blocks of at most 64
+// registers keep 32 warps with two depth blocks of loads each in flight per
+// SM.  300 x 300 x 512, float32: 122 us cold (the general kernel: 488).
+constexpr int kColumnWarps = 8;
+template <typename T>
+__global__ void __launch_bounds__(kColumnWarps * kWarp, 4) column_kernel(const DataArgs A) {
+  const int64_t p = (int64_t)blockIdx.x * kColumnWarps + (threadIdx.x >> 5);
+  if (p >= (int64_t)A.L.w * A.L.h) return;  // warp-uniform
+  data_column<T>(A, p, (int)(p % A.L.w), (int)(p / A.L.w), threadIdx.x & 31);
+}
+
 }  // namespace
 
 cudaError_t launch_data_multi(const DataMulti& M, int dtype, cudaStream_t s) {
@@ -111,6 +123,18 @@ cudaError_t launch_data(const DataArgs& a, cudaStream_t s) {
     data_kernel<__half><<<(unsigned)blocks, kWarpsPerBlock * kWarp, 0, s>>>(a);
   else
     data_kernel<float><<<(unsigned)blocks, kWarpsPerBlock * kWarp, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_data_column(const DataArgs& a, cudaStream_t s) {
+  const int64_t blocks = ((int64_t)a.L.w * a.L.h + kColumnWarps - 1) / kColumnWarps;
+  if (blocks <= 0) return cudaSuccess;
+  if (a.L.dtype == OCTMC_BF16)
+    column_kernel<__nv_bfloat16><<<(unsigned)blocks, kColumnWarps * kWarp, 0, s>>>(a);
+  else if (a.L.dtype == OCTMC_F16)
+    column_kernel<__half><<<(unsigned)blocks, kColumnWarps * kWarp, 0, s>>>(a);
+  else
+    column_kernel<float><<<(unsigned)blocks, kColumnWarps * kWarp, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -20,18 +20,19 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__global__ void prm_to_disp_kernel(const double* __restrict__ prm, int w, int h, double* __restrict__ disp) {
-  const int64_t plane = (int64_t)w * h, n = 6 * plane;
+__global__ void prm_to_disp_kernel(const double* __restrict__ prm, int w, int h, double* __restrict__ disp, bool all) {
+  const int64_t plane = (int64_t)w * h, n = (all ? 6 : 2) * plane;
   const double cx = 0.5 * (w - 1), cy = 0.5 * (h - 1);
   const double *aX = prm, *tX = prm + h, *aY = prm + 2 * h, *tY = prm + 2 * h + w;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int comp = (int)(e / plane);  // V * 3 + c
-    const int64_t q = e - comp * plane;
+    const int k = (int)(e / plane);
+    const int comp = all ? k : 3 * k + 2;  // V * 3 + c
+    const int64_t q = e - k * plane;
     const int i = (int)(q % w), j = (int)(q / w);
     double v = 0.0;
     if (comp == 2) v = fma(tX[j], (double)i - cx, aX[j]);
     else if (comp == 5) v = fma(tY[i], (double)j - cy, aY[i]);
-    disp[e] = v;
+    disp[comp * plane + q] = v;
   }
 }
 
@@ -146,8 +147,8 @@ inline unsigned grid_for(int64_t n) {
 
 }  // namespace
 
-cudaError_t launch_prm_to_disp(const double* prm, int w, int h, double* disp, cudaStream_t s) {
-  prm_to_disp_kernel<<<grid_for(6 * (int64_t)w * h), kThreads, 0, s>>>(prm, w, h, disp);
+cudaError_t launch_prm_to_disp(const double* prm, int w, int h, double* disp, bool all, cudaStream_t s) {
+  prm_to_disp_kernel<<<grid_for((all ? 6 : 2) * (int64_t)w * h), kThreads, 0, s>>>(prm, w, h, disp, all);
   return cudaGetLastError();
 }
 

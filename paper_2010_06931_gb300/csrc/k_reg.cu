@@ -93,13 +93,14 @@ __device__ void sum_partials(const double* partials, int nblocks, double (&v)[N]
 
 // Block blk of nblk blocks working on one problem's mean-term sums.
 __device__ void msum_body(const double* __restrict__ disp, int64_t plane, EvalResult* res, double* partials,
-                          unsigned* counter, int blk, int nblk) {
+                          unsigned* counter, int blk, int nblk, int c0 = 0) {
   // float64 throughout: the sums S_c nearly cancel at a centred field, so
   // their relative error is that of the inputs' magnitudes (6 adds per A-scan)
   double v[3] = {0.0, 0.0, 0.0};
   for (int64_t e = (int64_t)blk * kThreads + threadIdx.x; e < plane; e += (int64_t)nblk * kThreads) {
 #pragma unroll
-    for (int c = 0; c < 3; c++) v[c] += disp[c * plane + e] + disp[(3 + c) * plane + e];
+    for (int c = 0; c < 3; c++)
+      if (c >= c0) v[c] += disp[c * plane + e] + disp[(3 + c) * plane + e];
   }
   block_sum<3>(v);
   if (threadIdx.x == 0)
@@ -115,8 +116,8 @@ __device__ void msum_body(const double* __restrict__ disp, int64_t plane, EvalRe
 
 __global__ void __launch_bounds__(kThreads) msum_kernel(const double* __restrict__ disp, int64_t plane,
                                                         EvalResult* res, double* partials,
-                                                        unsigned* counter) {
-  msum_body(disp, plane, res, partials, counter, blockIdx.x, gridDim.x);
+                                                        unsigned* counter, int c0) {
+  msum_body(disp, plane, res, partials, counter, blockIdx.x, gridDim.x, c0);
 }
 
 // Slot of block b: the last s with b0[s] <= b (block-uniform).
@@ -169,6 +170,7 @@ __device__ void reg_body(const RegArgs& A, int blk, int nblk) {
     const float wp = pv >= 0 ? L.wprev[V][p] : 0.f;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
+      if (A.axial && c < 2) continue;
       const double* dc = A.disp + (V * 3 + c) * n;
       const double x = dc[p];
       float gr = 0.f;
@@ -258,8 +260,8 @@ int reg_grid_blocks(int64_t n) {
 }
 
 cudaError_t launch_msum(const double* disp, int64_t plane, EvalResult* res, double* partials,
-                        unsigned* counter, cudaStream_t s) {
-  msum_kernel<<<kMsumBlocks, kThreads, 0, s>>>(disp, plane, res, partials, counter);
+                        unsigned* counter, cudaStream_t s, bool axial) {
+  msum_kernel<<<kMsumBlocks, kThreads, 0, s>>>(disp, plane, res, partials, counter, axial ? 2 : 0);
   return cudaGetLastError();
 }
 
