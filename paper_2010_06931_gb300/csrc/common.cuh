@@ -33,12 +33,14 @@ __device__ __forceinline__ void keys_weights(float t, float w[4], float dw[4]) {
 // v_b + (v_{b+1} - v_b) (3 t^2 - 2 t^3), edge samples replicated.  It is C^1
 // and never leaves the range of its two nodes, so delta (Eq. 8) stays within
 // [0, delta_0] next to invalid B-scans.
-__device__ __forceinline__ void validity_hermite(const float* v, int n, int b, float t, float* val,
-                                                 float* dval) {
-  const float p0 = v[clampi(b, n)], p1 = v[clampi(b + 1, n)];
+__device__ __forceinline__ void hermite01(float p0, float p1, float t, float* val, float* dval) {
   const float dp = p1 - p0;
   *val = fmaf(dp, (t * t) * fmaf(-2.0f, t, 3.0f), p0);
   *dval = dp * (6.0f * t) * (1.0f - t);
+}
+__device__ __forceinline__ void validity_hermite(const float* v, int n, int b, float t, float* val,
+                                                 float* dval) {
+  hermite01(v[clampi(b, n)], v[clampi(b + 1, n)], t, val, dval);
 }
 
 // Exact split of u = off + v, v a double given by its bit pattern and off an
@@ -274,6 +276,8 @@ struct RegArgs {
   const double* eta_dev;  // if not null: eta is read here
   bool axial;             // only the axial components (the transverse ones of disp are 0)
   EvalResult* result;     // device
+  double* terms_out;      // may be null: the 6 terms, in device memory of the caller
+  EvalResult* host_out;   // may be null: the result in pinned host memory
   double* partials;       // [grid][8] scratch
   unsigned* counter;      // zero-initialised, reset by the last block
   SolveState* ctl;        // may be null: the line-search decision of a device-resident solve

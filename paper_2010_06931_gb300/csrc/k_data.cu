@@ -18,9 +18,9 @@
 // unaligned bytes; spilled registers cost it one more each) and by the
 // latency of its misses, so both fewer registers (more spills) and fewer
 // warps lose.  300 x 300 x 512, float32, data kernel alone: 64 registers
-// 517 us, 72 registers 488 us, 80 registers 500 us (529 us with depth-paired
-// multiply-adds and a per-lane prologue; bfloat16 535 -> 469 us; 64^3 19.2 ->
-// 16.6 us).
+// 488 us, 72 registers 466 us, 80 registers about 480 us (529 us with
+// depth-paired multiply-adds and a per-lane prologue and epilogue; bfloat16
+// 535 -> 455 us; 64^3 19.2 -> 13.4 us).
 //
 // The per-A-scan prologue (coordinate split, 24 weight pairs, 16 offsets) is
 // evaluated by a few lanes into a table in shared memory and the epilogue's 7
@@ -88,7 +88,7 @@ data_multi_kernel(const __grid_constant__ DataMulti M) {
 // The data term of a field without transverse displacement: one warp per
 // A-scan, two columns read once.  Bound by HBM; 8-warp blocks of at most 64
 // registers keep 32 warps with two depth blocks of loads each in flight per
-// SM.  300 x 300 x 512, float32: 122 us cold (the general kernel: 488).
+// SM.  300 x 300 x 512, float32: 122 us cold (the general kernel: 466).
 constexpr int kColumnWarps = 8;
 template <typename T>
 __global__ void __launch_bounds__(kColumnWarps * kWarp, 4) column_kernel(const DataArgs A) {

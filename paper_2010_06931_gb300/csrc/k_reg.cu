@@ -31,25 +31,37 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMsumBlocks = 152;
 constexpr int kMaxRegBlocks = 608;
 
-// Sum of v[c] over the block, result valid in thread 0 (fixed tree).
-template <int N>
-__device__ void block_sum(double (&v)[N]) {
-  __shared__ double sm[N][kWarps];
+// Sums of v[c] over the block, results valid in thread 0 (fixed tree: a
+// butterfly over the lanes, then one over the warps).  N = 4 (pad with 0): the
+// first two butterfly stages keep half of the values each and the warps'
+// totals of all values go through one butterfly, which pairs the same terms
+// with 6 + 3 float64 additions per lane instead of 20 + 12 (one such
+// instruction holds the SM's float64 pipe for 16 cycles).
+__device__ void block_sum(double (&v)[4]) {
+  static_assert(kWarps == 8, "one lane per value and warp below");
+  __shared__ double sm[4][kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int c = 0; c < N; c++) {
-    const double s = warp_sum(v[c]);
-    if (lane == 0) sm[c][warp] = s;
+  for (int n = 2; n >= 1; n >>= 1) {
+    const bool up = (lane & (8 * n)) != 0;
+#pragma unroll
+    for (int c = 0; c < n; c++) {
+      const double send = up ? v[c] : v[c + n];
+      const double keep = up ? v[c + n] : v[c];
+      v[c] = keep + __shfl_xor_sync(0xffffffffu, send, 8 * n);
+    }
   }
+  double s = v[0];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((lane & 7) == 0) sm[lane >> 3][warp] = s;  // lane 8 c: value c
   __syncthreads();
   if (warp == 0) {
+    double t = sm[lane >> 3][lane & 7];
 #pragma unroll
-    for (int c = 0; c < N; c++) {
-      double s = lane < kWarps ? sm[c][lane] : 0.0;
+    for (int o = kWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
 #pragma unroll
-      for (int o = kWarps / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      v[c] = s;
-    }
+    for (int c = 0; c < 4; c++) v[c] = __shfl_sync(0xffffffffu, t, 8 * c);
   }
   __syncthreads();
 }
@@ -82,13 +94,13 @@ __device__ bool last_block(unsigned* counter, int nblk) {
 // The last block adds partials[b * N + c] over the blocks b, in a fixed
 // strided order per thread followed by block_sum.  Result in thread 0.
 template <int N>
-__device__ void sum_partials(const double* partials, int nblocks, double (&v)[N]) {
+__device__ void sum_partials(const double* partials, int nblocks, double (&v)[4]) {
 #pragma unroll
-  for (int c = 0; c < N; c++) v[c] = 0.0;
+  for (int c = 0; c < 4; c++) v[c] = 0.0;
   for (int b = threadIdx.x; b < nblocks; b += kThreads)
 #pragma unroll
     for (int c = 0; c < N; c++) v[c] += partials[b * N + c];
-  block_sum<N>(v);
+  block_sum(v);
 }
 
 // Block blk of nblk blocks working on one problem's mean-term sums.
@@ -96,13 +108,13 @@ __device__ void msum_body(const double* __restrict__ disp, int64_t plane, EvalRe
                           unsigned* counter, int blk, int nblk, int c0 = 0) {
   // float64 throughout: the sums S_c nearly cancel at a centred field, so
   // their relative error is that of the inputs' magnitudes (6 adds per A-scan)
-  double v[3] = {0.0, 0.0, 0.0};
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
   for (int64_t e = (int64_t)blk * kThreads + threadIdx.x; e < plane; e += (int64_t)nblk * kThreads) {
 #pragma unroll
     for (int c = 0; c < 3; c++)
       if (c >= c0) v[c] += disp[c * plane + e] + disp[(3 + c) * plane + e];
   }
-  block_sum<3>(v);
+  block_sum(v);
   if (threadIdx.x == 0)
     for (int c = 0; c < 3; c++) partials[blk * 3 + c] = v[c];
   if (last_block(counter, nblk)) {
@@ -200,33 +212,38 @@ __device__ void reg_body(const RegArgs& A, int blk, int nblk) {
     v[2] += widen_exact(r);
     v[3] += gd;
   }
-  block_sum<4>(v);
-  gmx = block_max(gmx);
+  block_sum(v);
+  if (A.ctl) gmx = block_max(gmx);  // only the solve's stopping test reads it
   if (threadIdx.x == 0) {
     for (int c = 0; c < 4; c++) A.partials[blk * 4 + c] = v[c];
-    A.partials[4 * nblk + blk] = __longlong_as_double((long long)gmx);
+    if (A.ctl) A.partials[4 * nblk + blk] = __longlong_as_double((long long)gmx);
   }
   if (last_block(A.counter, nblk)) {
     sum_partials<4>(A.partials, nblk, v);
     unsigned long long m = 0ull;
-    for (int b = threadIdx.x; b < nblk; b += kThreads)
-      m = max(m, (unsigned long long)__double_as_longlong(A.partials[4 * nblk + b]));
-    m = block_max(m);
+    if (A.ctl) {
+      for (int b = threadIdx.x; b < nblk; b += kThreads)
+        m = max(m, (unsigned long long)__double_as_longlong(A.partials[4 * nblk + b]));
+      m = block_max(m);
+    }
     if (threadIdx.x == 0) {
       const double* ms = A.result->msum;
       const double M = A.mu * (ms[0] * ms[0] + ms[1] * ms[1] + ms[2] * ms[2]);
       EvalResult* res = A.result;
-      res->terms[0] = v[0];
-      res->terms[1] = v[1];
       const double eta = A.eta_dev ? *A.eta_dev : A.eta;
       const double R = (double)L.d * v[2];
-      res->terms[2] = R;
-      res->terms[3] = M;
-      res->terms[4] = eta * v[0] + v[1] / eta + A.alpha * R + M;
-      res->terms[5] = eta;
+      const double t[6] = {v[0], v[1], R, M, eta * v[0] + v[1] / eta + A.alpha * R + M, eta};
+      const double f = t[4];
+#pragma unroll
+      for (int c = 0; c < 6; c++) {
+        res->terms[c] = t[c];
+        if (A.terms_out) A.terms_out[c] = t[c];
+        if (A.host_out) A.host_out->terms[c] = t[c];  // visible to the host once the stream is synchronised
+      }
       res->gdir = v[3];
+      if (A.host_out) A.host_out->gdir = v[3];
       *A.counter = 0u;
-      if (A.ctl) ls_decide(A.ctl, res->terms[4], v[3], __longlong_as_double((long long)m), A.h_branch, A.h_while);
+      if (A.ctl) ls_decide(A.ctl, f, v[3], __longlong_as_double((long long)m), A.h_branch, A.h_while);
     }
   }
 }
