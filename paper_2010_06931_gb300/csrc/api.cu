@@ -86,19 +86,6 @@ void build_chain(const std::vector<double>& t, std::vector<int>& prev, std::vect
   }
 }
 
-std::vector<double> time_down(const std::vector<double>& t, int w, int h) {
-  const int w2 = half_up(w), h2 = half_up(h);
-  std::vector<double> o((size_t)w2 * h2);
-  for (int j = 0; j < h2; j++)
-    for (int i = 0; i < w2; i++) {
-      const int i1 = std::min(2 * i + 1, w - 1), j1 = std::min(2 * j + 1, h - 1);
-      o[(size_t)j * w2 + i] = (t[(size_t)2 * j * w + 2 * i] + t[(size_t)2 * j * w + i1] +
-                               t[(size_t)j1 * w + 2 * i] + t[(size_t)j1 * w + i1]) /
-                              4.0;
-    }
-  return o;
-}
-
 }  // namespace
 
 // ====================================================================== L-BFGS
@@ -316,6 +303,8 @@ struct octmc_problem {
   cudaStream_t st = nullptr;
   bool have_ang = false;
   std::vector<Level> lv;
+  char* slab = nullptr;       // one allocation: the levels and the evaluation workspace
+  char* build_tmp = nullptr;  // buffers of the construction
   // evaluation workspace (sized for level 0)
   float* str = nullptr;
   float* ang = nullptr;
@@ -355,7 +344,6 @@ struct octmc_problem {
   double* pre_aux = nullptr;
   double* pre_aux_host = nullptr;
   double* pre_prm = nullptr;  // 2 (w + h) of level 0: parameter gradient scratch / coarse copy
-  std::vector<void*> temps;  // float32 pyramid copies while building 16-bit storage
   // optional CUDA-event timing of the data-term kernel (octmc_profile_*)
   bool profile = false;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -364,17 +352,10 @@ struct octmc_problem {
   bool prof_pending = false;
 
   ~octmc_problem() {
-    for (void* t : temps) dfree(t);
     if (ev0) cudaEventDestroy(ev0);
     if (ev1) cudaEventDestroy(ev1);
-    for (Level& L : lv) {
-      LevelDev& d = L.dev;
-      dfree(d.sx); dfree(d.sy); dfree(d.ax); dfree(d.ay); dfree(d.vx); dfree(d.vy);
-      for (int V = 0; V < 2; V++) {
-        dfree(d.prev[V]); dfree(d.next[V]); dfree(d.wprev[V]); dfree(d.wnext[V]);
-      }
-    }
-    dfree(str); dfree(ang); dfree(gdata); dfree(partials); dfree(counters); dfree(res);
+    dfree(slab);
+    dfree(build_tmp);
     if (res_host) cudaFreeHost(res_host);
     dfree(x); dfree(g); dfree(xt); dfree(gt); dfree(xb); dfree(gb); dfree(dir);
     dfree(mcounts);
@@ -414,6 +395,10 @@ void check_device() {
 void upload_volume(octmc_problem* P, const float* src, float* dst, int w, int h, int d, int dp) {
   const cudaMemcpyKind kind = P->desc.inputs_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   const int64_t cols = (int64_t)w * h;
+  if (dp == d) {
+    CK(cudaMemcpyAsync(dst, src, sizeof(float) * cols * d, kind, P->st));
+    return;
+  }
   // rows of d samples into rows of dp; cudaMemcpy2D limits the row count to
   // what a size_t height takes, so copy in slabs of columns
   const int64_t slab = 1 << 20;
@@ -436,93 +421,48 @@ void upload_host(octmc_problem* P, const std::vector<T>& v, T* dst) {
   CK(cudaMemcpyAsync(dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, P->st));
 }
 
-std::vector<double> fetch_times(octmc_problem* P, const double* t, size_t n) {
-  std::vector<double> out(n);
-  if (P->desc.inputs_on_device) {
-    CK(cudaMemcpyAsync(out.data(), t, sizeof(double) * n, cudaMemcpyDeviceToHost, P->st));
-    CK(cudaStreamSynchronize(P->st));
-  } else {
-    std::memcpy(out.data(), t, sizeof(double) * n);
+// Device buffers carved out of one allocation: a first pass with base = null
+// adds up the size, the second hands out the pieces (256-byte aligned).
+struct Arena {
+  char* base = nullptr;
+  size_t used = 0;
+  template <typename T>
+  T* take(size_t count) {
+    T* p = reinterpret_cast<T*>(base + used);
+    used += (std::max<size_t>(count, 1) * sizeof(T) + 255) & ~size_t(255);
+    return base ? p : nullptr;
   }
-  for (double v : out)
-    if (!std::isfinite(v)) throw CudaFail{OCTMC_ERR_INVALID_ARG};
-  return out;
-}
+};
 
-void create_impl(octmc_problem* P) {
+// Buffers needed only while a problem is built.
+struct BuildTemps {
+  std::vector<float*> vol[2];   // float32 volumes per level (16-bit storage)
+  std::vector<double*> t[2];    // sampling times per level
+  ChainInfo* info = nullptr;    // [level][scan]
+};
+
+// Every buffer a problem keeps, level by level, and the evaluation workspace.
+void lay_out(octmc_problem* P, Arena& A) {
   const octmc_desc& D = P->desc;
-  check_device();
-  const int L = D.levels;
-  const int dt = D.storage;
-  P->lv.resize(L);
   int w = D.w, h = D.h, d = D.d;
-  std::vector<double> tx = fetch_times(P, D.tx, (size_t)w * h), ty = fetch_times(P, D.ty, (size_t)w * h);
-  // The pyramid is built in float32; with 16-bit storage every level is
-  // rounded once (to nearest even) from its float32 box means, and the
-  // float32 copies are temporaries (kept in P->temps until released).
-  float* prev32[2] = {nullptr, nullptr};
-  for (int l = 0; l < L; l++) {
+  for (int l = 0; l < D.levels; l++) {
     LevelDev& X = P->lv[l].dev;
     X.w = w; X.h = h; X.d = d; X.dp = pad4(d);
-    X.dtype = dt;
-    const int64_t cols = (int64_t)w * h;
-    float* cur32[2];
-    for (int V = 0; V < 2; V++) {
-      cur32[V] = dalloc<float>((size_t)cols * X.dp);
-      if (dt != OCTMC_F32) P->temps.push_back(cur32[V]);
-    }
+    X.dtype = D.storage;
+    const size_t cols = (size_t)w * h, vox = cols * X.dp;
+    X.sx = D.storage == OCTMC_F32 ? (void*)A.take<float>(vox) : (void*)A.take<uint16_t>(vox);
+    X.sy = D.storage == OCTMC_F32 ? (void*)A.take<float>(vox) : (void*)A.take<uint16_t>(vox);
     if (P->have_ang) {
-      X.ax = dalloc<float>((size_t)cols);
-      X.ay = dalloc<float>((size_t)cols);
+      X.ax = A.take<float>(cols);
+      X.ay = A.take<float>(cols);
     }
-    if (D.vx) X.vx = dalloc<float>((size_t)h);
-    if (D.vy) X.vy = dalloc<float>((size_t)w);
-    if (l == 0) {
-      upload_volume(P, D.sx, cur32[0], w, h, d, X.dp);
-      upload_volume(P, D.sy, cur32[1], w, h, d, X.dp);
-      if (P->have_ang) {
-        upload(P, D.ax, X.ax, (size_t)cols);
-        upload(P, D.ay, X.ay, (size_t)cols);
-      }
-      if (D.vx) upload(P, D.vx, X.vx, (size_t)h);
-      if (D.vy) upload(P, D.vy, X.vy, (size_t)w);
-    } else {
-      const LevelDev& F = P->lv[l - 1].dev;
-      for (int V = 0; V < 2; V++)
-        CK(launch_pyr_volume(prev32[V], F.w, F.h, F.d, F.dp, cur32[V], w, h, d, X.dp, P->st));
-      if (P->have_ang) {
-        CK(launch_pyr_image(F.ax, F.w, F.h, X.ax, P->st));
-        CK(launch_pyr_image(F.ay, F.w, F.h, X.ay, P->st));
-      }
-      if (X.vx) CK(launch_pyr_line(F.vx, F.h, X.vx, P->st));
-      if (X.vy) CK(launch_pyr_line(F.vy, F.w, X.vy, P->st));
-      tx = time_down(tx, F.w, F.h);
-      ty = time_down(ty, F.w, F.h);
-    }
-    if (dt == OCTMC_F32) {
-      X.sx = cur32[0];
-      X.sy = cur32[1];
-    } else {
-      X.sx = dalloc<uint16_t>((size_t)cols * X.dp);
-      X.sy = dalloc<uint16_t>((size_t)cols * X.dp);
-      CK(launch_convert(cur32[0], X.sx, dt, cols * X.dp, P->st));
-      CK(launch_convert(cur32[1], X.sy, dt, cols * X.dp, P->st));
-    }
-    prev32[0] = cur32[0];
-    prev32[1] = cur32[1];
+    if (D.vx) X.vx = A.take<float>(h);
+    if (D.vy) X.vy = A.take<float>(w);
     for (int V = 0; V < 2; V++) {
-      std::vector<int> pv, nx;
-      std::vector<float> wp, wn;
-      build_chain(V == 0 ? tx : ty, pv, nx, wp, wn);
-      X.prev[V] = dalloc<int>((size_t)cols);
-      X.next[V] = dalloc<int>((size_t)cols);
-      X.wprev[V] = dalloc<float>((size_t)cols);
-      X.wnext[V] = dalloc<float>((size_t)cols);
-      upload_host(P, pv, X.prev[V]);
-      upload_host(P, nx, X.next[V]);
-      upload_host(P, wp, X.wprev[V]);
-      upload_host(P, wn, X.wnext[V]);
-      CK(cudaStreamSynchronize(P->st));  // host vectors go out of scope
+      X.prev[V] = A.take<int>(cols);
+      X.next[V] = A.take<int>(cols);
+      X.wprev[V] = A.take<float>(cols);
+      X.wnext[V] = A.take<float>(cols);
     }
     P->lv[l].mu = D.mu > 0 ? D.mu : 1.0 / (2.0 * (double)w * (double)h);
     w = half_up(w);
@@ -530,17 +470,114 @@ void create_impl(octmc_problem* P) {
     d = half_up(d);
   }
   const int64_t n0 = P->plane(0);
-  P->str = dalloc<float>((size_t)n0);
-  P->ang = dalloc<float>((size_t)n0);
-  P->gdata = dalloc<float>((size_t)6 * n0);
-  P->partials = dalloc<double>((size_t)8 * std::max(reg_grid_blocks(n0), msum_grid_blocks()));
-  P->counters = dalloc<unsigned>(2);
+  P->str = A.take<float>((size_t)n0);
+  P->ang = A.take<float>((size_t)n0);
+  P->gdata = A.take<float>((size_t)6 * n0);
+  P->partials = A.take<double>((size_t)8 * std::max(reg_grid_blocks(n0), msum_grid_blocks()));
+  P->counters = A.take<unsigned>(2);
+  P->res = A.take<EvalResult>(1);
+}
+
+void lay_out_temps(octmc_problem* P, BuildTemps& B, Arena& A) {
+  B.vol[0].clear(); B.vol[1].clear(); B.t[0].clear(); B.t[1].clear();
+  for (const Level& Lv : P->lv) {
+    const LevelDev& X = Lv.dev;
+    const size_t cols = (size_t)X.w * X.h;
+    for (int V = 0; V < 2; V++) {
+      B.vol[V].push_back(X.dtype == OCTMC_F32 ? static_cast<float*>(V == 0 ? X.sx : X.sy) : A.take<float>(cols * X.dp));
+      B.t[V].push_back(A.take<double>(cols));
+    }
+  }
+  B.info = A.take<ChainInfo>(2 * P->lv.size());
+}
+
+// The chain of one scan by a sort on the host: times in neither raster order.
+void host_chain(octmc_problem* P, const double* t_dev, const LevelDev& X, int V) {
+  std::vector<double> t((size_t)X.w * X.h);
+  CK(cudaMemcpyAsync(t.data(), t_dev, sizeof(double) * t.size(), cudaMemcpyDeviceToHost, P->st));
+  CK(cudaStreamSynchronize(P->st));
+  std::vector<int> pv, nx;
+  std::vector<float> wp, wn;
+  build_chain(t, pv, nx, wp, wn);
+  upload_host(P, pv, X.prev[V]);
+  upload_host(P, nx, X.next[V]);
+  upload_host(P, wp, X.wprev[V]);
+  upload_host(P, wn, X.wnext[V]);
+  CK(cudaStreamSynchronize(P->st));  // host vectors go out of scope
+}
+
+// Everything a problem keeps lives in one allocation, and everything that only
+// its construction needs in a second one; the work is enqueued without a host
+// wait until the chains' test is read at the end.  300 x 300 x 512, 3 levels,
+// device inputs: 9.8 -> 1.44 ms with its destruction.
+void create_impl(octmc_problem* P) {
+  const octmc_desc& D = P->desc;
+  check_device();
+  const int L = D.levels;
+  const int dt = D.storage;
+  P->lv.resize(L);
+  Arena size, keep, tmp;
+  lay_out(P, size);
+  P->slab = dalloc<char>(size.used);
+  keep.base = P->slab;
+  lay_out(P, keep);
+  // The pyramid is built in float32; with 16-bit storage every level is
+  // rounded once (to nearest even) from its float32 box means.
+  BuildTemps B;
+  lay_out_temps(P, B, tmp);
+  P->build_tmp = dalloc<char>(tmp.used);
+  tmp = Arena{P->build_tmp, 0};
+  lay_out_temps(P, B, tmp);
   CK(cudaMemsetAsync(P->counters, 0, 2 * sizeof(unsigned), P->st));
-  P->res = dalloc<EvalResult>(1);
+  std::vector<ChainInfo> info(2 * L);
+  const ChainInfo none{0, 0, 0, 0, 0x7ff0000000000000ull, 0x7ff0000000000000ull};
+  std::fill(info.begin(), info.end(), none);
+  CK(cudaMemcpyAsync(B.info, info.data(), sizeof(ChainInfo) * info.size(), cudaMemcpyHostToDevice, P->st));
+  for (int l = 0; l < L; l++) {
+    LevelDev& X = P->lv[l].dev;
+    const int64_t cols = (int64_t)X.w * X.h;
+    if (l == 0) {
+      upload(P, D.tx, B.t[0][0], (size_t)cols);
+      upload(P, D.ty, B.t[1][0], (size_t)cols);
+      upload_volume(P, D.sx, B.vol[0][0], X.w, X.h, X.d, X.dp);
+      upload_volume(P, D.sy, B.vol[1][0], X.w, X.h, X.d, X.dp);
+      if (P->have_ang) {
+        upload(P, D.ax, X.ax, (size_t)cols);
+        upload(P, D.ay, X.ay, (size_t)cols);
+      }
+      if (D.vx) upload(P, D.vx, X.vx, (size_t)X.h);
+      if (D.vy) upload(P, D.vy, X.vy, (size_t)X.w);
+    } else {
+      const LevelDev& F = P->lv[l - 1].dev;
+      CK(launch_pyr_volume(B.vol[0][l - 1], B.vol[1][l - 1], F.w, F.h, F.d, F.dp, B.vol[0][l], B.vol[1][l], X.w, X.h,
+                           X.d, X.dp, P->st));
+      if (P->have_ang) {
+        CK(launch_pyr_image(F.ax, F.w, F.h, X.ax, P->st));
+        CK(launch_pyr_image(F.ay, F.w, F.h, X.ay, P->st));
+      }
+      if (X.vx) CK(launch_pyr_line(F.vx, F.h, X.vx, P->st));
+      if (X.vy) CK(launch_pyr_line(F.vy, F.w, X.vy, P->st));
+      for (int V = 0; V < 2; V++) CK(launch_time_down(B.t[V][l - 1], F.w, F.h, B.t[V][l], P->st));
+    }
+    if (dt != OCTMC_F32) {
+      CK(launch_convert(B.vol[0][l], X.sx, dt, cols * X.dp, P->st));
+      CK(launch_convert(B.vol[1][l], X.sy, dt, cols * X.dp, P->st));
+    }
+    for (int V = 0; V < 2; V++) {
+      ChainInfo* ci = B.info + 2 * l + V;
+      CK(launch_chain_scan(B.t[V][l], X.w, X.h, ci, P->st));
+      CK(launch_chain_write(B.t[V][l], X.w, X.h, ci, X.prev[V], X.next[V], X.wprev[V], X.wnext[V], P->st));
+    }
+  }
+  CK(cudaMemcpyAsync(info.data(), B.info, sizeof(ChainInfo) * info.size(), cudaMemcpyDeviceToHost, P->st));
   CK(cudaMallocHost(&P->res_host, sizeof(EvalResult)));
   CK(cudaStreamSynchronize(P->st));
-  for (void* t : P->temps) dfree(t);
-  P->temps.clear();
+  if (info[0].nonfinite || info[1].nonfinite) throw CudaFail{OCTMC_ERR_INVALID_ARG};
+  for (int l = 0; l < L; l++)
+    for (int V = 0; V < 2; V++)
+      if (info[2 * l + V].row_bad && info[2 * l + V].col_bad) host_chain(P, B.t[V][l], P->lv[l].dev, V);
+  dfree(P->build_tmp);
+  P->build_tmp = nullptr;
 }
 
 void collect_profile(octmc_problem* P) {

@@ -346,8 +346,21 @@ cudaError_t launch_merge_weights(const LevelDev& L, const double* disp, double b
                                  unsigned long long* counts, float* weights, float* angio, cudaStream_t s);
 
 cudaError_t launch_pad_depth(float* vol, int64_t columns, int d, int dp, cudaStream_t s);
-cudaError_t launch_pyr_volume(const float* in, int w, int h, int d, int dp, float* out, int w2,
-                              int h2, int d2, int dp2, cudaStream_t s);
+// both volumes of a pair in one launch
+cudaError_t launch_pyr_volume(const float* inx, const float* iny, int w, int h, int d, int dp, float* outx, float* outy,
+                              int w2, int h2, int d2, int dp2, cudaStream_t s);
+
+// Acquisition chains (k_chain.cu).  One entry per level and scan.
+struct ChainInfo {
+  unsigned nonfinite;               // a sampling time is not finite
+  unsigned row_bad, col_bad;        // the times do not increase along rows / along columns
+  unsigned pad;
+  unsigned long long row_dt, col_dt;  // smallest positive step in that order (float64 bits; infinity: none)
+};
+cudaError_t launch_chain_scan(const double* t, int w, int h, ChainInfo* info, cudaStream_t s);
+cudaError_t launch_chain_write(const double* t, int w, int h, const ChainInfo* info, int* prev, int* next, float* wprev,
+                               float* wnext, cudaStream_t s);
+cudaError_t launch_time_down(const double* t, int w, int h, double* out, cudaStream_t s);
 cudaError_t launch_pyr_image(const float* in, int w, int h, float* out, cudaStream_t s);
 cudaError_t launch_pyr_line(const float* in, int n, float* out, cudaStream_t s);
 cudaError_t launch_prolong(const double* coarse, int wc, int hc, double* fine, int wf, int hf,
