@@ -288,6 +288,19 @@ int octmc_enface(const float *octa_dev, const float *oct_dev, int w, int h, int 
                  const float *v_dev, double q_lo, double q_hi, double thresh, double t_oct, float *enface_dev,
                  float *filtered_dev, double *info_host, void *stream);
 
+/* octmc_enface with the caller's scratch instead of the stream-ordered
+ * allocator's (whose volumes are mapped and unmapped on every call):
+ * workspace_dev is device memory of at least octmc_enface_workspace(...) bytes,
+ * 256-byte aligned, used on `stream` until the call returns; its contents do
+ * not matter.  INVALID_ARG if it is too small or misaligned. */
+int octmc_enface_ws(const float *octa_dev, const float *oct_dev, int w, int h, int d, int fast_axis,
+                    const float *v_dev, double q_lo, double q_hi, double thresh, double t_oct, float *enface_dev,
+                    float *filtered_dev, double *info_host, void *workspace_dev, int64_t workspace_bytes,
+                    void *stream);
+/* Bytes of scratch octmc_enface_ws needs for a scan of this size; -1 for an
+ * invalid size. */
+int64_t octmc_enface_workspace(int w, int h, int d, int fast_axis);
+
 /* Copies pyramid data of `level` to device buffers (any may be NULL):
  * sx/sy as float32 [h][w][d], ax/ay [h][w], vx[h], vy[w]. */
 int octmc_level_data(const octmc_problem *p, int level, float *sx, float *sy, float *ax, float *ay,

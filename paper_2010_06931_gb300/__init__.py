@@ -320,9 +320,12 @@ def enface(octa, oct, fast_axis, v, q_lo=0.05, q_hi=0.95, thresh=0.1, t_oct=None
                                  or not filtered.is_cuda or not filtered.is_contiguous()):
         raise ValueError("filtered must be a contiguous float32 CUDA tensor of the volume's shape")
     info = (C.c_double * 4)()
-    N.check(N.lib().octmc_enface(_ptr(A), _ptr(S), w, h, d, int(fast_axis), _ptr(vv), float(q_lo), float(q_hi),
-                                 float(thresh), float("nan") if t_oct is None else float(t_oct), _ptr(E),
-                                 _ptr(filtered), info, _stream_ptr()), "octmc_enface")
+    # scratch from PyTorch's caching allocator; the call waits for the stream, so it may go when it returns
+    nws = max(0, int(N.lib().octmc_enface_workspace(w, h, d, int(fast_axis))))
+    ws = torch.empty(nws, dtype=torch.uint8, device="cuda")
+    N.check(N.lib().octmc_enface_ws(_ptr(A), _ptr(S), w, h, d, int(fast_axis), _ptr(vv), float(q_lo), float(q_hi),
+                                    float(thresh), float("nan") if t_oct is None else float(t_oct), _ptr(E),
+                                    _ptr(filtered), info, _ptr(ws), nws, _stream_ptr()), "octmc_enface")
     return E, dict(p_lo=info[0], p_hi=info[1], t_oct=info[2], kept=int(info[3]))
 
 

@@ -67,6 +67,9 @@ _SIGS = {
     "octmc_saccade_validity": (C.c_int, [C.c_void_p] + [C.c_int] * 4 + [C.c_void_p] * 3),
     "octmc_enface": (C.c_int, [C.c_void_p, C.c_void_p] + [C.c_int] * 4 + [C.c_void_p] + [C.c_double] * 4
                      + [C.c_void_p] * 4),
+    "octmc_enface_ws": (C.c_int, [C.c_void_p, C.c_void_p] + [C.c_int] * 4 + [C.c_void_p] + [C.c_double] * 4
+                        + [C.c_void_p] * 4 + [C.c_int64, C.c_void_p]),
+    "octmc_enface_workspace": (C.c_int64, [C.c_int] * 4),
     "octmc_lbfgs_create": (C.c_int, [C.c_int64, C.c_int, C.c_void_p, C.POINTER(C.c_void_p)]),
     "octmc_lbfgs_destroy": (None, [C.c_void_p]),
     "octmc_lbfgs_push": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p]),

@@ -149,6 +149,33 @@ __device__ __forceinline__ float narrow_trunc(double x) {
   return __uint_as_float(sign | ((unsigned)ef << 23) | mant);
 }
 
+// The exact sum of 8 floats as s + e, s the rounded sum (Knuth's two-sum).
+// Float64 additions run at 1/64 of the float rate on this GPU; this takes 42
+// float additions for 8.  True where the sum is exact: the non-zero magnitudes
+// lie within 2^16 of one another and between 2^-60 and 1e37, so the errors,
+// multiples of the smallest sample's last bit and below 2^21 of them in all,
+// add exactly in float.  NaN and infinities fail the test on s.
+__device__ __forceinline__ bool exact_sum8(const float x[8], float* sum, float* err) {
+  float mx = 0.f, mn = INFINITY;
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    const float a = fabsf(x[k]);
+    mx = fmaxf(mx, a);
+    if (a > 0.f) mn = fminf(mn, a);
+  }
+  float s = x[0], e = 0.f;
+#pragma unroll
+  for (int k = 1; k < 8; k++) {
+    const float t = __fadd_rn(s, x[k]);
+    const float b = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x[k], b)));
+    s = t;
+  }
+  *sum = s;
+  *err = e;
+  return mn * 65536.0f >= mx && mn >= 8.7e-19f && mx < 1e37f && fabsf(s) < 1e38f;
+}
+
 // Deterministic warp sum (xor butterfly; every lane ends with the total).
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

@@ -67,33 +67,12 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(const float4* __restr
   }
 }
 
-// Mean of 8 samples: the sum added in double (in the order of x), rounded once
-// to float.  Double additions are 1/64 of the float rate here, so where the
-// samples' magnitudes lie within 2^16 of one another (and none is subnormal)
-// the sum is formed in float with its rounding errors (Knuth's two-sum): the
-// partial sums fit 24 + 16 + 3 bits and the errors, multiples of the smallest
-// sample's last bit below 2^-20 of the largest, add exactly in float, so the
-// one rounding s + e is that of the exact sum -- which the double sum (43 of 53
-// bits) is too.
+// Mean of 8 samples: the sum added in double (in the order of x) or, with the
+// same result, exactly in float (exact_sum8: the double sum needs 43 of 53
+// bits there), rounded once to float.
 __device__ __forceinline__ float mean8(const float x[8]) {
-  float mx = 0.f, mn = INFINITY;
-#pragma unroll
-  for (int k = 0; k < 8; k++) {
-    const float a = fabsf(x[k]);
-    mx = fmaxf(mx, a);
-    if (a > 0.f) mn = fminf(mn, a);
-  }
-  // NaN samples fail the comparisons through the sum below being non-finite
-  float s = x[0], e = 0.f;
-#pragma unroll
-  for (int k = 1; k < 8; k++) {
-    const float t = __fadd_rn(s, x[k]);
-    const float bb = __fsub_rn(t, s);
-    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(x[k], bb)));
-    s = t;
-  }
-  // mn >= 2^-60: the errors are normal floats; a finite s also excludes NaN and infinities
-  if (mn * 65536.0f >= mx && mn >= 8.7e-19f && fabsf(s) < 1e38f && mx < 1e37f) return __fmul_rn(__fadd_rn(s, e), 0.125f);
+  float s, e;
+  if (exact_sum8(x, &s, &e)) return __fmul_rn(__fadd_rn(s, e), 0.125f);
   double q = 0.0;
 #pragma unroll
   for (int k = 0; k < 8; k += 2) q += (double)x[k] + (double)x[k + 1];
