@@ -48,50 +48,77 @@ __device__ double block_sum_d(double v, double* sm) {
   return t;
 }
 
+// Sums of 6 values over the block, in every thread (v[6], v[7] = 0): a
+// reduce-scatter with a butterfly's pairing, then the warps' totals in warp
+// order by one thread per value; two barriers for all six.
+__device__ void block_sum6(double (&v)[8], double* sm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int n = 4; n >= 1; n >>= 1) {
+    const bool up = (lane & (4 * n)) != 0;
+#pragma unroll
+    for (int k = 0; k < n; k++) {
+      const double send = up ? v[k] : v[k + n];
+      const double keep = up ? v[k + n] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * n);
+    }
+  }
+  double t = v[0];
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  if ((lane & 3) == 0) sm[(lane >> 2) * (kThreads / 32) + warp] = t;  // lane 4 k: value k
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    double s = 0.0;
+    for (int i = 0; i < kThreads / 32; i++) s += sm[threadIdx.x * (kThreads / 32) + i];
+    sm[8 * (kThreads / 32) + threadIdx.x] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 6; k++) v[k] = sm[8 * (kThreads / 32) + k];
+}
+
 // Block b < h: X B-scan (row) b; block h + b: Y B-scan (column) b.  Writes
 // d f / d a and d f / d t of the B-scan (field gradient reduced along the
-// fast axis, plus the tilt term's part); block 0 writes T to *T_out.
+// fast axis, plus the tilt term's part); block 0 writes T to *T_out.  Bound by
+// the latency of its float64 sums: one reduction of all six instead of six in
+// a row, 600 B-scans: 41 -> 16 us.
 __global__ void __launch_bounds__(kThreads) grad_to_prm_kernel(const double* __restrict__ g, int w, int h,
                                                                const double* __restrict__ prm,
                                                                double* __restrict__ gprm, double* T_out) {
-  __shared__ double sm[kThreads / 32];
+  __shared__ double sm[8 * (kThreads / 32) + 6];
   const int64_t plane = (int64_t)w * h;
   const bool isX = blockIdx.x < (unsigned)h;
   const int b = isX ? blockIdx.x : blockIdx.x - h;
   const int nf = isX ? w : h;
   const double c = 0.5 * (nf - 1);
   const double* gz = g + (isX ? 2 : 5) * plane;
-  double ga = 0.0, gt = 0.0;
+  double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // ga, gt, sX, sY, sT, nT
   for (int f = threadIdx.x; f < nf; f += kThreads) {
-    const double v = isX ? gz[(int64_t)b * w + f] : gz[(int64_t)f * w + b];
-    ga += v;
-    gt = fma(v, (double)f - c, gt);
+    const double x = isX ? gz[(int64_t)b * w + f] : gz[(int64_t)f * w + b];
+    v[0] += x;
+    v[1] = fma(x, (double)f - c, v[1]);
   }
-  ga = block_sum_d(ga, sm);
-  gt = block_sum_d(gt, sm);
   // the tilt functionals (same order in every block)
   const double cx = 0.5 * (w - 1), cy = 0.5 * (h - 1);
-  double sX = 0.0, sY = 0.0, sT = 0.0, nT = 0.0;
   for (int k = threadIdx.x; k < h; k += kThreads) {
     const double t = prm[h + k], o = (double)k - cy;
-    sX += t;
-    sT = fma(t, o, sT);
-    nT = fma(o, o, nT);
+    v[2] += t;
+    v[4] = fma(t, o, v[4]);
+    v[5] = fma(o, o, v[5]);
   }
   for (int k = threadIdx.x; k < w; k += kThreads) {
     const double t = prm[2 * h + w + k], o = (double)k - cx;
-    sY += t;
-    sT = fma(t, o, sT);
-    nT = fma(o, o, nT);
+    v[3] += t;
+    v[4] = fma(t, o, v[4]);
+    v[5] = fma(o, o, v[5]);
   }
-  sX = block_sum_d(sX, sm);
-  sY = block_sum_d(sY, sm);
-  sT = block_sum_d(sT, sm);
-  nT = block_sum_d(nT, sm);
-  const double vx = ((double)w * w - 1.0) / 12.0, vy = ((double)h * h - 1.0) / 12.0;
-  const double lx = 2.0 * w * vx / h, ly = 2.0 * h * vy / w;
-  const double lt = nT > 0.0 ? 2.0 * w * h * vx * vy / (nT * nT) : 0.0;
+  block_sum6(v, sm);
   if (threadIdx.x == 0) {
+    const double ga = v[0], gt = v[1], sX = v[2], sY = v[3], sT = v[4], nT = v[5];
+    const double vx = ((double)w * w - 1.0) / 12.0, vy = ((double)h * h - 1.0) / 12.0;
+    const double lx = 2.0 * w * vx / h, ly = 2.0 * h * vy / w;
+    const double lt = nT > 0.0 ? 2.0 * w * h * vx * vy / (nT * nT) : 0.0;
     if (isX) {
       gprm[b] = ga;
       gprm[h + b] = gt + 2.0 * lx * sX + 2.0 * lt * sT * ((double)b - cy);
