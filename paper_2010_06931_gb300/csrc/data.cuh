@@ -61,47 +61,38 @@ __device__ __forceinline__ float warp_totals8(float v[8], int lane) {
   return t;
 }
 
-// The data-term computation of output A-scan p (i, j) by one warp, with `tab`
-// (2 entries) the warp's shared-memory table.  Lane 4 v returns output v: v = 0 the
-// structural term, v = 1 + 3 V + c the gradient component c of scan V; lane
-// 28 the angiographic term.
-template <typename T>
-__device__ __forceinline__ float data_value(const DataArgs& A, VolTab* tab, int64_t p, int i, int j, int lane) {
-  const LevelDev& L = A.L;
-  Vol VX, VY;
-  setup_pair(VX, VY, tab, A.disp, (int64_t)L.w * L.h, p, i, j, L, lane);
-
-  const float inv_eps = 1.0f / A.eps_h;
-  const bool ssd = (A.loss == OCTMC_LOSS_SSD);
-  // L, then the x, y, z sums of dL dI for X and for Y
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  // outputs inside the volume from this lane's first output on (none for the halo lanes)
-  int left = (lane >= 1 && lane <= kOutLanes) ? L.d - 4 * (lane - 1) : 0;
-  for (int kb = 0; kb < L.d; kb += kOutPerIter, left -= kOutPerIter) {
-    float2 XZ[4], XG[4], YZ[4], YG[4];
-    sample_block<T>(VX, kb, lane, L.dp, XZ, XG);
-    sample_block<T>(VY, kb, lane, L.dp, YZ, YG);
-    auto add = [&](int o) {
-      float Lv, dL;
-      loss_grad(XZ[o].x - YZ[o].x, inv_eps, ssd, &Lv, &dL);
-      acc[0] += Lv;
-      float2 t = ffma2(both(dL), XG[o], make_float2(acc[1], acc[2]));
-      acc[1] = t.x; acc[2] = t.y;
-      acc[3] = fmaf(dL, XZ[o].y, acc[3]);
-      t = ffma2(both(dL), YG[o], make_float2(acc[4], acc[5]));
-      acc[4] = t.x; acc[5] = t.y;
-      acc[6] = fmaf(dL, YZ[o].y, acc[6]);
-    };
-    // outputs outside the volume add nothing, whatever their lanes hold
-    if (left >= 4) {
+// Adds one depth block to the sums acc: L, then the x, y, z sums of dL dI for X
+// and for Y.  left: outputs inside the volume from the lane's first output on;
+// those outside add nothing, whatever their lanes hold.
+__device__ __forceinline__ void add_block(float acc[8], const float2 XZ[4], const float2 XG[4], const float2 YZ[4],
+                                          const float2 YG[4], int left, float inv_eps, bool ssd) {
+  auto add = [&](int o) {
+    float Lv, dL;
+    loss_grad(XZ[o].x - YZ[o].x, inv_eps, ssd, &Lv, &dL);
+    acc[0] += Lv;
+    float2 t = ffma2(both(dL), XG[o], make_float2(acc[1], acc[2]));
+    acc[1] = t.x; acc[2] = t.y;
+    acc[3] = fmaf(dL, XZ[o].y, acc[3]);
+    t = ffma2(both(dL), YG[o], make_float2(acc[4], acc[5]));
+    acc[4] = t.x; acc[5] = t.y;
+    acc[6] = fmaf(dL, YZ[o].y, acc[6]);
+  };
+  if (left >= 4) {
 #pragma unroll
-      for (int o = 0; o < 4; o++) add(o);
-    } else if (left > 0) {
-      add(0);
-      if (left > 1) add(1);
-      if (left > 2) add(2);
-    }
+    for (int o = 0; o < 4; o++) add(o);
+  } else if (left > 0) {
+    add(0);
+    if (left > 1) add(1);
+    if (left > 2) add(2);
   }
+}
+
+// The outputs of an A-scan from its depth sums: lane 4 v returns output v: v = 0
+// the structural term, v = 1 + 3 V + c the gradient component c of scan V; lane
+// 28 the angiographic term.
+__device__ __forceinline__ float data_outputs(const DataArgs& A, const VolTab* tab, const Vol& VX, const Vol& VY,
+                                              float acc[8], float inv_eps, bool ssd, int lane) {
+  const LevelDev& L = A.L;
   // the loads of the epilogue together, before the sums: this lane's tap of the
   // en-face images (lanes 0..15 A^X, 16..31 A^Y) and, in lanes 0..3, the
   // validity nodes around the displaced positions.  (Issued ahead of the depth
@@ -164,6 +155,29 @@ __device__ __forceinline__ float data_value(const DataArgs& A, VolTab* tab, int6
   if (v == 0) out = (1.0f - delta) * Lsum;
   if (v == 7) out = delta * d * La;
   return out;
+}
+
+// The data-term computation of output A-scan p (i, j) by one warp from the
+// volumes in global memory, with `tab` (2 entries) the warp's shared-memory
+// table; the value of this lane's output (see data_outputs).
+template <typename T>
+__device__ __forceinline__ float data_value(const DataArgs& A, VolTab* tab, int64_t p, int i, int j, int lane) {
+  const LevelDev& L = A.L;
+  Vol VX, VY;
+  setup_pair(VX, VY, tab, A.disp, (int64_t)L.w * L.h, p, i, j, L, lane);
+  const Sampler WX(tab[0]), WY(tab[1]);
+  const float inv_eps = 1.0f / A.eps_h;
+  const bool ssd = (A.loss == OCTMC_LOSS_SSD);
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  // outputs inside the volume from this lane's first output on (none for the halo lanes)
+  int left = (lane >= 1 && lane <= kOutLanes) ? L.d - 4 * (lane - 1) : 0;
+  for (int kb = 0; kb < L.d; kb += kOutPerIter, left -= kOutPerIter) {
+    float2 XZ[4], XG[4], YZ[4], YG[4];
+    sample_block<T>(VX, WX, kb, lane, L.dp, XZ, XG);
+    sample_block<T>(VY, WY, kb, lane, L.dp, YZ, YG);
+    add_block(acc, XZ, XG, YZ, YG, left, inv_eps, ssd);
+  }
+  return data_outputs(A, tab, VX, VY, acc, inv_eps, ssd, lane);
 }
 
 // ---- fields without transverse displacement (the axial prealignment)
@@ -278,16 +292,20 @@ __device__ __forceinline__ void data_column(const DataArgs& A, int64_t p, int i,
   if (A.grad && lane >= 1) A.grad[(lane == 1 ? 2 : 5) * nasc + p] = lane == 1 ? cs * gx : -cs * gy;
 }
 
-// Output A-scan p = (i, j) by one warp: data_value written out.
-template <typename T>
-__device__ __forceinline__ void data_ascan(const DataArgs& A, VolTab* tab, int64_t p, int i, int j, int lane) {
-  const float out = data_value<T>(A, tab, p, i, j, lane);
+// This lane's output of A-scan p written out.
+__device__ __forceinline__ void data_store(const DataArgs& A, int64_t p, float out, int lane) {
   const int64_t nasc = (int64_t)A.L.w * A.L.h;
   const int v = lane >> 2;
   if (lane & 3) return;
   if (v == 0) A.str_out[p] = out;
   else if (v == 7) A.ang_out[p] = out;
   else if (A.grad) A.grad[(int64_t)(v - 1) * nasc + p] = out;
+}
+
+// Output A-scan p = (i, j) by one warp: data_value written out.
+template <typename T>
+__device__ __forceinline__ void data_ascan(const DataArgs& A, VolTab* tab, int64_t p, int i, int j, int lane) {
+  data_store(A, p, data_value<T>(A, tab, p, i, j, lane), lane);
 }
 
 }  // namespace

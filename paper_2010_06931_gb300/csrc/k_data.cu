@@ -13,14 +13,14 @@
 // Mapping: one warp per output A-scan; the sampling and its lane layout are
 // described in sample.cuh.  A block's 4 warps take a tile of 2 x 2
 // neighbouring A-scans (their 4 x 4 neighbourhoods overlap, which the L1 cache
-// turns into hits).  At 72 registers 7 blocks (28 warps) run per SM: the
-// kernel is bound by the L1 data pipe (volume loads, 5 wavefronts per 512
-// unaligned bytes; spilled registers cost it one more each) and by the
-// latency of its misses, so both fewer registers (more spills) and fewer
-// warps lose.  300 x 300 x 512, float32, data kernel alone: 64 registers
-// 488 us, 72 registers 466 us, 80 registers about 480 us (529 us with
-// depth-paired multiply-adds and a per-lane prologue and epilogue; bfloat16
-// 535 -> 455 us; 64^3 19.2 -> 13.4 us).
+// turns into hits).  At 64 registers 8 blocks (32 warps) run per SM: the
+// kernel is bound by the L1 data pipe (80 % busy: volume loads, 5 wavefronts
+// per 512 unaligned bytes, then shuffles and spills) and by the latency of its
+// misses, so both more registers (fewer warps) and fewer (more spills) lose.
+// 300 x 300 x 512, float32, data kernel alone: 48 / 56 / 64 / 72 / 80 registers
+// 462 / 438 / 420 / 449 / 437 us, 8- and 16-warp blocks 423 and 437 us (529 us
+// with depth-paired multiply-adds, spilled weights and a per-lane prologue and
+// epilogue; bfloat16 535 -> 395 us; 64^3 19.2 -> 14.0 us).
 //
 // The per-A-scan prologue (coordinate split, 24 weight pairs, 16 offsets) is
 // evaluated by a few lanes into a table in shared memory and the epilogue's 7
@@ -37,7 +37,7 @@ namespace octmc {
 namespace {
 
 #ifndef OCTMC_DATA_MINB
-#define OCTMC_DATA_MINB 7
+#define OCTMC_DATA_MINB 8
 #endif
 #ifndef OCTMC_DTILE_X
 #define OCTMC_DTILE_X 2
@@ -88,7 +88,7 @@ data_multi_kernel(const __grid_constant__ DataMulti M) {
 // The data term of a field without transverse displacement: one warp per
 // A-scan, two columns read once.  Bound by HBM; 8-warp blocks of at most 64
 // registers keep 32 warps with two depth blocks of loads each in flight per
-// SM.  300 x 300 x 512, float32: 122 us cold (the general kernel: 466).
+// SM.  300 x 300 x 512, float32: 122 us cold (the general kernel: 420).
 constexpr int kColumnWarps = 8;
 template <typename T>
 __global__ void __launch_bounds__(kColumnWarps * kWarp, 4) column_kernel(const DataArgs A) {

@@ -21,7 +21,6 @@
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
-#include <stddef.h>
 
 #include "common.cuh"
 
@@ -44,33 +43,21 @@ struct alignas(16) VolTab {
 
 struct Vol {
   const void* base;    // the volume; addressed in groups of 4 samples
-  unsigned tab;        // shared-memory address of its VolTab
   int q, r;            // floor(dz) = 4 q + r, 0 <= r < 4
   int bx, by;          // floor of the transverse coordinates
   float ts;            // the fraction along the scan's slow axis (y for X, x for Y), Eq. 7
 };
-
-// Table reads.  Volatile: each is one broadcast load at the place of use, so
-// the table is not kept in (or spilled from) the registers of the depth loop.
-__device__ __forceinline__ void lds4(unsigned addr, float2& a, float2& b) {
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a.x), "=f"(a.y), "=f"(b.x), "=f"(b.y) : "r"(addr));
-}
-__device__ __forceinline__ void lds2(unsigned addr, float2& a) {
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(a.x), "=f"(a.y) : "r"(addr));
-}
-__device__ __forceinline__ void lds4u(unsigned addr, unsigned u[4]) {
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]) : "r"(addr));
-}
 
 // Coordinate split of the 6 displacement values of A-scan (i, j) by lanes
 // 0..5 (lane = 3 V + c): floor(u) and the float fraction for u = i + dx and
 // u = j + dy clamped to [-4, n + 3] (beyond that every tap is an edge sample)
 // and u = dz clamped to +-(d + 8) (all depth taps are then edge samples).
 // Integer arithmetic only (split_exact).  The lane then evaluates the 4
-// weights of its component, and lanes 0..15 the neighbour offsets, once per
-// A-scan; the warp reads them back from shared memory.
-__device__ __forceinline__ void setup_pair(Vol& VX, Vol& VY, VolTab* tab, const double* disp, int64_t nasc, int64_t p,
-                                           int i, int j, const LevelDev& L, int lane) {
+// weights of its component into the table, once per A-scan.  Returns, in lanes
+// 0..15, the clamped index of a neighbour row or column: lanes 0..7 volume X,
+// 8..15 volume Y; 4 rows, then 4 columns.
+__device__ __forceinline__ int split_pair(Vol& VX, Vol& VY, VolTab* tab, const double* disp, int64_t nasc, int64_t p,
+                                          int i, int j, const LevelDev& L, int lane) {
   int b = 0;
   float t = 0.f;
   const int c = lane < 3 ? lane : lane - 3;
@@ -100,19 +87,20 @@ __device__ __forceinline__ void setup_pair(Vol& VX, Vol& VY, VolTab* tab, const 
   VX.r = zx & 3;
   VY.q = zy >> 2;
   VY.r = zy & 3;
-  if (lane < 16) {  // lanes 0..7: volume X, 8..15: volume Y; 4 rows, then 4 columns
-    const unsigned nq = (unsigned)(L.dp >> 2);
-    const int a = lane & 3;
-    const bool isY = lane >= 8;
-    const unsigned off = (lane & 4) ? (unsigned)clampi((isY ? VY.bx : VX.bx) - 1 + a, L.w) * nq
-                                    : (unsigned)clampi((isY ? VY.by : VX.by) - 1 + a, L.h) * (unsigned)L.w * nq;
-    tab[isY ? 1 : 0].off[lane & 7] = off;
-  }
-  __syncwarp();
-  VX.tab = (unsigned)__cvta_generic_to_shared(tab);
-  VY.tab = VX.tab + (unsigned)sizeof(VolTab);
   VX.base = L.sx;
   VY.base = L.sy;
+  const bool isY = lane >= 8;
+  const int a = (lane & 3) - 1;
+  return (lane & 4) ? clampi((isY ? VY.bx : VX.bx) + a, L.w) : clampi((isY ? VY.by : VX.by) + a, L.h);
+}
+
+// The same with the table's offsets into the volumes in global memory.
+__device__ __forceinline__ void setup_pair(Vol& VX, Vol& VY, VolTab* tab, const double* disp, int64_t nasc, int64_t p,
+                                           int i, int j, const LevelDev& L, int lane) {
+  const int n = split_pair(VX, VY, tab, disp, nasc, p, i, j, L, lane);
+  const unsigned nq = (unsigned)(L.dp >> 2);
+  if (lane < 16) tab[lane >> 3].off[lane & 7] = (unsigned)n * ((lane & 4) ? nq : (unsigned)L.w * nq);
+  __syncwarp();
 }
 
 // Four consecutive samples (one aligned group) widened to float: float32
@@ -203,60 +191,84 @@ __device__ __forceinline__ void axial(const float T[4], const float2 Txy[4], con
   }
 }
 
+// The table's weights and offsets as warp-uniform values.  A warp reduction
+// delivers its result in a uniform register, which the packed multiply-add
+// takes as an operand, so the 48 weights and 16 offsets of an A-scan hardly need
+// the vector registers that limit the warps per SM: 64 registers hold all of
+// them with about 110 bytes spilled.  Read from shared memory in every depth
+// block instead (72 registers) they cost the L1 data pipe, the kernel's bound:
+// 300 x 300 x 512, float32 466 -> 420 us, bfloat16 446 -> 395 us; 237 x 301 x
+// 465, float16 358 -> 332 us.
+struct Sampler {
+  float2 wx[4], wy[4], wz[4];
+  unsigned roff[4], coff[4];
+  static __device__ __forceinline__ unsigned uniform(unsigned v) { return __reduce_or_sync(kFull, v); }
+  static __device__ __forceinline__ float2 uniform(float2 v) {
+    return make_float2(__uint_as_float(uniform(__float_as_uint(v.x))), __uint_as_float(uniform(__float_as_uint(v.y))));
+  }
+  __device__ __forceinline__ explicit Sampler(const VolTab& T) {
+#pragma unroll
+    for (int a = 0; a < 4; a++) {
+      wx[a] = uniform(T.wx[a]);
+      wy[a] = uniform(T.wy[a]);
+      wz[a] = uniform(T.wz[a]);
+      roff[a] = uniform(T.off[a]);
+      coff[a] = uniform(T.off[4 + a]);
+    }
+  }
+};
+
 // (I, dI/dz) and (dI/dx, dI/dy) of one volume at the lane's 4 outputs.  qk:
 // first input depth of the lane's group (samples, may lie outside the
-// volume); qc: index of that group's (clamped) samples in the volume.
-template <typename S>
-__device__ __forceinline__ void sample_group(const Vol& V, int qk, unsigned qc, int dp, float2 Iz[4], float2 Ixy[4]) {
+// volume); load(b, a): the group's (clamped) samples in neighbour row b, column
+// a.
+template <typename Load>
+__device__ __forceinline__ void sample_group(const Sampler& W, int r, int qk, int dp, Load&& load, float2 Iz[4],
+                                             float2 Ixy[4]) {
   float T[4];
-  float2 Txy[4], wx[4], wz[4];
-  unsigned coff[4], roff[4];
-  lds4u(V.tab + offsetof(VolTab, off) + 16, coff);
-  lds4u(V.tab + offsetof(VolTab, off), roff);
-  lds4(V.tab + offsetof(VolTab, wx), wx[0], wx[1]);
-  lds4(V.tab + offsetof(VolTab, wx) + 16, wx[2], wx[3]);
+  float2 Txy[4];
 #pragma unroll
   for (int b = 0; b < 4; b++) {
     float2 U[4];  // (d/dx, value) of row b
-    float2 wy;
-    lds2(V.tab + offsetof(VolTab, wy) + 8 * b, wy);
 #pragma unroll
     for (int a = 0; a < 4; a++) {
-      const float4 f = load4<S>(V.base, roff[b] + coff[a] + qc);
+      const float4 f = load(b, a);
       const float s[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
-      for (int k = 0; k < 4; k++) U[k] = a == 0 ? fmul2(wx[0], both(s[k])) : ffma2(wx[a], both(s[k]), U[k]);
+      for (int k = 0; k < 4; k++) U[k] = a == 0 ? fmul2(W.wx[0], both(s[k])) : ffma2(W.wx[a], both(s[k]), U[k]);
     }
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-      Txy[k] = b == 0 ? fmul2(wy, U[k]) : ffma2(wy, U[k], Txy[k]);
-      T[k] = b == 0 ? wy.x * U[k].y : fmaf(wy.x, U[k].y, T[k]);
+      Txy[k] = b == 0 ? fmul2(W.wy[0], U[k]) : ffma2(W.wy[b], U[k], Txy[k]);
+      T[k] = b == 0 ? W.wy[0].x * U[k].y : fmaf(W.wy[b].x, U[k].y, T[k]);
     }
   }
   // groups entirely before sample 0 / after the last sample hold the edge value
-  if (qk < 0) {
+  if (__any_sync(kFull, (unsigned)qk >= (unsigned)dp)) {
+    if (qk < 0) {
 #pragma unroll
-    for (int k = 1; k < 4; k++) { T[k] = T[0]; Txy[k] = Txy[0]; }
-  } else if (qk >= dp) {
+      for (int k = 1; k < 4; k++) { T[k] = T[0]; Txy[k] = Txy[0]; }
+    } else if (qk >= dp) {
 #pragma unroll
-    for (int k = 0; k < 3; k++) { T[k] = T[3]; Txy[k] = Txy[3]; }
+      for (int k = 0; k < 3; k++) { T[k] = T[3]; Txy[k] = Txy[3]; }
+    }
   }
-  lds4(V.tab + offsetof(VolTab, wz), wz[0], wz[1]);
-  lds4(V.tab + offsetof(VolTab, wz) + 16, wz[2], wz[3]);
-  switch (V.r) {
-    case 0: axial<0>(T, Txy, wz, Iz, Ixy); break;
-    case 1: axial<1>(T, Txy, wz, Iz, Ixy); break;
-    case 2: axial<2>(T, Txy, wz, Iz, Ixy); break;
-    default: axial<3>(T, Txy, wz, Iz, Ixy); break;
+  switch (r) {
+    case 0: axial<0>(T, Txy, W.wz, Iz, Ixy); break;
+    case 1: axial<1>(T, Txy, W.wz, Iz, Ixy); break;
+    case 2: axial<2>(T, Txy, W.wz, Iz, Ixy); break;
+    default: axial<3>(T, Txy, W.wz, Iz, Ixy); break;
   }
 }
 
-// The same at the lane's 4 outputs of the depth block starting at kb.
+// The same at the lane's 4 outputs of the depth block starting at kb, from the
+// volume in global memory.
 template <typename S>
-__device__ __forceinline__ void sample_block(const Vol& V, int kb, int lane, int dp, float2 Iz[4], float2 Ixy[4]) {
+__device__ __forceinline__ void sample_block(const Vol& V, const Sampler& W, int kb, int lane, int dp, float2 Iz[4],
+                                             float2 Ixy[4]) {
   const int qk = kb + 4 * V.q + 4 * (lane - 1);  // first input depth of the lane's group
   const unsigned qc = (unsigned)(min(max(qk, 0), dp - 4) >> 2);
-  sample_group<S>(V, qk, qc, dp, Iz, Ixy);
+  sample_group(W, V.r, qk, dp, [&](int b, int a) { return load4<S>(V.base, W.roff[b] + W.coff[a] + qc); }, Iz, Ixy);
 }
 
 }  // namespace
