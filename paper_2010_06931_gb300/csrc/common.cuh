@@ -258,8 +258,6 @@ struct __align__(16) SolveState {  // 16-byte aligned: copied to shared memory w
   int k, spare, ncand;
   int order[kMaxM + 1];
   int cand[kMaxM + 1];
-  double SY[(kMaxM + 1) * (kMaxM + 1)];
-  double YY[(kMaxM + 1) * (kMaxM + 1)];
   double sg[kMaxM + 1], yg[kMaxM + 1];
   double gg, gmax;
   // direction: dir = cg g + sum_j coef[j] h_j, h_j = S[hid[j] / 2] (even) or Y[hid[j] / 2] (odd)
@@ -268,6 +266,10 @@ struct __align__(16) SolveState {  // 16-byte aligned: copied to shared memory w
   int hid[2 * kMaxM + 2];
   double coef[2 * kMaxM + 2];
   double dots[2 * (2 * kMaxM + 2) + 3];
+  // last: the products kernel works on a shared-memory copy of everything
+  // before these and reads the k x k entries it needs from here
+  alignas(16) double SY[(kMaxM + 1) * (kMaxM + 1)];
+  double YY[(kMaxM + 1) * (kMaxM + 1)];
 };
 
 // Configuration of a level solve, set on the device at the level's start.

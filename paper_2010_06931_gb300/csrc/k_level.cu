@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kLThreads, 1) level_kernel(const __grid_consta
   __shared__ const double* s_hp[kMaxVec];
   __shared__ double s_cf[kMaxVec];
   __shared__ VolTab tab[kLWarps][2];
-  copy_state<kLThreads>(&sS, A.S);
+  copy_state<kLThreads, sizeof(SolveState)>(&sS, A.S);
   __syncthreads();
   const int G = gridDim.x, B = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kLThreads, 1) level_kernel(const __grid_consta
         for (int t = 0; t < ncand; t++) sS.cand[t] = (t < nstored) ? sS.order[t] : sS.spare;
       }
       __syncthreads();
-      after_products(&sS, alg);
+      after_products(&sS, sS.SY, sS.YY, alg);
       __syncthreads();
     }
   }
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kLThreads, 1) level_kernel(const __grid_consta
     for (int64_t e = (int64_t)B * kLThreads + tid; e < n; e += (int64_t)G * kLThreads) V.x[e] = xs[e];
   }
   __syncthreads();
-  if (B == 0) copy_state<kLThreads>(A.S, &sS);
+  if (B == 0) copy_state<kLThreads, sizeof(SolveState)>(A.S, &sS);
 }
 
 // One grid barrier that waits for `extra` more blocks than the grid has:

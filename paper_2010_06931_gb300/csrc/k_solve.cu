@@ -22,9 +22,9 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kChunk = 20;             // history vectors per block row
+constexpr int kChunk = 6;              // history vectors per block row
 constexpr int kMaxVec = 2 * kMaxM + 2; // history vectors of one product pass
-constexpr int kVals = 64;              // per-thread partial sums of the products (2 kChunk + 2, padded)
+constexpr int kVals = 32;              // per-thread partial sums of the products (2 kChunk + 2, padded)
 
 __device__ __forceinline__ const double* hvec(const HistSet& H, int id) {
   return (id & 1) ? H.Y[id >> 1] : H.S[id >> 1];
@@ -222,13 +222,16 @@ __device__ __forceinline__ void dots_pass(const double* const* h, int kn, int cs
 
 // Products of the candidate history vectors (the stored pairs and, after an
 // accepted step, the new one) with the probes y_new (accepted step only) and
-// the gradient; g . g.  Grid (G, rows): G blocks (one per SM) split the
+// the gradient; g . g.  6 vectors per row, so that several blocks share an SM
+// and one reduce-scatter of 32 sums ends a block (20 per row and one block per
+// SM: 58 -> 52 us per iteration of a 64^3 solve, level 0 of 300 x 300 x 512 84 ->
+// 76 us).  Grid (G, rows): G blocks (one per SM) split the
 // elements into contiguous shares, rows cover the problem's longest history
-// (block (bx, r) takes candidates r*20 .. r*20+19; rows beyond this step's
+// (block (bx, r) takes candidates r*6 .. r*6+5; rows beyond this step's
 // candidates only arrive).  Within a block the float64 partial sums go
 // through the reduce-scatter above and a fixed sum over the warps; the last
 // block to finish adds the block partials (fixed order) and runs the algebra.
-__global__ void __launch_bounds__(kThreads, 1) dots_kernel(SolveState* S, const HistSet H, const SolveVecs V,
+__global__ void __launch_bounds__(kThreads, 2) dots_kernel(SolveState* S, const HistSet H, const SolveVecs V,
                                                            double* partials, unsigned* counter) {
   __shared__ double sm[kVals * kWarps];
   __shared__ bool is_last;
@@ -278,11 +281,9 @@ __global__ void __launch_bounds__(kThreads, 1) dots_kernel(SolveState* S, const 
   } else {
     dots_pass<false>(h, kn, -1, first, false, nullptr, gp, nullptr, nullptr, nullptr, nullptr, e0, e1, v);
   }
-  // warp totals: lane i holds values i and 32 + i
+  // warp totals: lane i holds value i
   const double t0 = warp_reduce_scatter32(v, lane);
-  const double t1 = warp_reduce_scatter32(v + 32, lane);
   sm[lane * kWarps + warp] = t0;
-  sm[(32 + lane) * kWarps + warp] = t1;
   __syncthreads();
   // block partials, outputs: [2v] = h_v . y, [2v+1] = h_v . g, [2K] = y . y, [2K+1] = g . g
   const int t = threadIdx.x;
@@ -302,10 +303,12 @@ __global__ void __launch_bounds__(kThreads, 1) dots_kernel(SolveState* S, const 
   if (!is_last) return;
   }
   __threadfence();
-  // the epilogue works on a shared-memory copy of the state: its serial parts
-  // would otherwise wait on L2 for every dependent access
-  __shared__ SolveState sS;
-  copy_state<kThreads>(&sS, S);
+  // the epilogue works on a shared-memory copy of the state (but for the
+  // products of the stored pairs): its serial parts would otherwise wait on L2
+  // for every dependent access
+  __shared__ __align__(16) unsigned char head[kStateHead];
+  SolveState& sS = *reinterpret_cast<SolveState*>(head);
+  copy_state<kThreads, kStateHead>(&sS, S);
   __syncthreads();
   const int nout = 2 * K + 2;
   for (int o = warp; o < nout; o += kWarps) {
@@ -318,13 +321,13 @@ __global__ void __launch_bounds__(kThreads, 1) dots_kernel(SolveState* S, const 
   if (threadIdx.x == 0) {
     *counter = 0u;
     sS.ncand = ncand;
-    for (int c = 0; c < ncand; c++) sS.cand[c] = (c < nstored) ? sS.order[c] : sS.spare;
   }
+  if (threadIdx.x < ncand) sS.cand[threadIdx.x] = (threadIdx.x < nstored) ? sS.order[threadIdx.x] : sS.spare;
   __syncthreads();
   __shared__ Algebra alg;
-  after_products(&sS, alg);
+  after_products(&sS, S->SY, S->YY, alg);
   __syncthreads();
-  copy_state<kThreads>(S, &sS);
+  copy_state<kThreads, kStateHead>(S, &sS);
 }
 
 __device__ __forceinline__ unsigned long long global_ns() {
