@@ -76,7 +76,7 @@ data_kernel(const DataArgs A) {
 template <typename T>
 __global__ void __launch_bounds__(kWarpsPerBlock * kWarp, OCTMC_DATA_MINB)
 data_multi_kernel(const __grid_constant__ DataMulti M) {
-  const DataArgs& A = M.da[blockIdx.y];
+  const DataArgs A = M.da[blockIdx.y];
   if ((int64_t)blockIdx.x >= direct_blocks(A.L.w, A.L.h)) return;
   __shared__ VolTab tab[kWarpsPerBlock][2];
   const int warp = threadIdx.x >> 5;
