@@ -202,8 +202,10 @@ __device__ __forceinline__ void axial_z(const float T[4], const float2 wz[4], fl
 
 __device__ __forceinline__ void column_filter(float4 f, int qk, int dp, int r, const float2 wz[4], float2 Iz[4]) {
   // groups entirely before sample 0 / after the last sample hold the edge value
-  if (qk < 0) f.y = f.z = f.w = f.x;
-  else if (qk >= dp) f.x = f.y = f.z = f.w;
+  if (__any_sync(kFull, (unsigned)qk >= (unsigned)dp)) {
+    if (qk < 0) f.y = f.z = f.w = f.x;
+    else if (qk >= dp) f.x = f.y = f.z = f.w;
+  }
   const float T[4] = {f.x, f.y, f.z, f.w};
   switch (r) {
     case 0: axial_z<0>(T, wz, Iz); break;

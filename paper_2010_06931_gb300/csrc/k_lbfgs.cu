@@ -15,7 +15,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kHistChunk = 20;         // history vectors per block row
+constexpr int kHistChunk = 6;          // history vectors per block row
 constexpr int kVals = 2 * kHistChunk + 2;  // sums per block row: h . q0, h . q1, then q0 . q0, q1 . q1
 
 __device__ bool last_block_2d(unsigned* counter) {
@@ -58,17 +58,17 @@ __device__ __forceinline__ double warp_reduce_scatter32(double* v, int lane) {
   return v[0];
 }
 
-// grid (G, rows): block (bx, r) takes history vectors r*20 .. r*20+19 over
-// a contiguous share of the n elements (one block per SM); row 0 also takes
+// grid (G, rows): block (bx, r) takes history vectors r*6 .. r*6+5 over
+// a contiguous share of the n elements; row 0 also takes
 // q0.q0, q1.q1 and max|q1| (the maximum on the bit patterns: exact, and NaN
 // wins).  Compiled for the probes that are given (kQ0, kQ1): bound by the
 // float64 pipe (0.50 T FMA/s measured), so the products with an absent probe
-// are left out.  16 vectors and one probe of 540000 elements: 86 -> 51 us.
+// are left out.  16 vectors and one probe of 540000 elements: 86 -> 48 us.
 // partials layout: [output][G].
 template <bool kQ0, bool kQ1>
-__global__ void __launch_bounds__(kThreads, 1) hist_dots_kernel(const HistDots D, int64_t n, double* partials,
+__global__ void __launch_bounds__(kThreads, 2) hist_dots_kernel(const HistDots D, int64_t n, double* partials,
                                                                 unsigned* counter, double* out) {
-  __shared__ double sm[64 * kWarps];
+  __shared__ double sm[32 * kWarps];
   __shared__ unsigned long long smx[kWarps];
   const int G = gridDim.x;
   const int k0 = blockIdx.y * kHistChunk;
@@ -77,10 +77,11 @@ __global__ void __launch_bounds__(kThreads, 1) hist_dots_kernel(const HistDots D
   const double* h[kHistChunk];
 #pragma unroll
   for (int k = 0; k < kHistChunk; k++) h[k] = (k < kn) ? D.h[k0 + k] : nullptr;
-  // v[2 k] = h_k . q0, v[2 k + 1] = h_k . q1, v[40] = q0 . q0, v[41] = q1 . q1
-  double v[64];
+  // v[2 k] = h_k . q0, v[2 k + 1] = h_k . q1, then q0 . q0, q1 . q1
+  static_assert(kVals <= 32, "one reduce-scatter");
+  double v[32];
 #pragma unroll
-  for (int k = 0; k < 64; k++) v[k] = 0.0;
+  for (int k = 0; k < 32; k++) v[k] = 0.0;
   unsigned long long mx = 0ull;
   const int64_t share = ((n + G - 1) / G + 31) / 32 * 32;
   const int64_t e0 = min(n, (int64_t)blockIdx.x * share), e1 = min(n, e0 + share);
@@ -104,9 +105,7 @@ __global__ void __launch_bounds__(kThreads, 1) hist_dots_kernel(const HistDots D
     }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const double t0 = warp_reduce_scatter32(v, lane), t1 = warp_reduce_scatter32(v + 32, lane);
-  sm[lane * kWarps + warp] = t0;
-  sm[(32 + lane) * kWarps + warp] = t1;
+  sm[lane * kWarps + warp] = warp_reduce_scatter32(v, lane);
   if (kQ1 && first) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -191,7 +190,7 @@ inline unsigned grid_for(int64_t n) {
 
 }  // namespace
 
-// One block per SM, fewer on short vectors.
+// Blocks per row: one per SM, fewer on short vectors.
 int hist_dots_blocks(int64_t n) {
   const int64_t b = (n + kThreads - 1) / kThreads;
   return (int)(b < 1 ? 1 : std::min<int64_t>(b, device_sm_count()));
