@@ -63,10 +63,13 @@ __device__ __forceinline__ double warp_reduce_scatter32(double* v, int lane) {
 // q0.q0, q1.q1 and max|q1| (the maximum on the bit patterns: exact, and NaN
 // wins).  Compiled for the probes that are given (kQ0, kQ1): bound by the
 // float64 pipe (0.50 T FMA/s measured), so the products with an absent probe
-// are left out.  16 vectors and one probe of 540000 elements: 86 -> 48 us.
+// are left out.  16 vectors and one probe of 540000 elements: 86 -> 48 us
+// with two blocks per SM; three, so that the three rows of 16 vectors are all
+// resident, take another 13 us (whole direction 99.7 -> 86.5 us; two rows of 8
+// or 10 vectors at two blocks per SM: 89.8, 86.9 us).
 // partials layout: [output][G].
 template <bool kQ0, bool kQ1>
-__global__ void __launch_bounds__(kThreads, 2) hist_dots_kernel(const HistDots D, int64_t n, double* partials,
+__global__ void __launch_bounds__(kThreads, 3) hist_dots_kernel(const HistDots D, int64_t n, double* partials,
                                                                 unsigned* counter, double* out) {
   __shared__ double sm[32 * kWarps];
   __shared__ unsigned long long smx[kWarps];

@@ -22,7 +22,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kChunk = 6;              // history vectors per block row
+constexpr int kChunk = 10;             // history vectors per block row
 constexpr int kMaxVec = 2 * kMaxM + 2; // history vectors of one product pass
 constexpr int kVals = 32;              // per-thread partial sums of the products (2 kChunk + 2, padded)
 
@@ -222,12 +222,15 @@ __device__ __forceinline__ void dots_pass(const double* const* h, int kn, int cs
 
 // Products of the candidate history vectors (the stored pairs and, after an
 // accepted step, the new one) with the probes y_new (accepted step only) and
-// the gradient; g . g.  6 vectors per row, so that several blocks share an SM
-// and one reduce-scatter of 32 sums ends a block (20 per row and one block per
-// SM: 58 -> 52 us per iteration of a 64^3 solve, level 0 of 300 x 300 x 512 84 ->
-// 76 us).  Grid (G, rows): G blocks (one per SM) split the
+// the gradient; g . g.  10 vectors per row: the 18 of a full history of 8
+// pairs are two rows, so all blocks are resident at two per SM, and one
+// reduce-scatter of 32 sums ends a block.  Time of a whole evaluation of a
+// one-level solve with 6 / 10 / 14 vectors per row: 59.3 / 60.3 / 61.3 us
+// (64 x 64 x 64), 78.9 / 71.3 / 72.7 us (75 x 75 x 128), 151.4 / 142.2 / 146.2 us
+// (150 x 150 x 256): three rows of 6 need a second wave of blocks as soon as a
+// row has one block per SM.  Grid (G, rows): G blocks (one per SM) split the
 // elements into contiguous shares, rows cover the problem's longest history
-// (block (bx, r) takes candidates r*6 .. r*6+5; rows beyond this step's
+// (block (bx, r) takes candidates r*10 .. r*10+9; rows beyond this step's
 // candidates only arrive).  Within a block the float64 partial sums go
 // through the reduce-scatter above and a fixed sum over the warps; the last
 // block to finish adds the block partials (fixed order) and runs the algebra.
