@@ -14,7 +14,6 @@ namespace octmc {
 namespace {
 
 constexpr int kThreads = 256;
-
 constexpr double kFix = 4294967296.0;  // 2^32
 
 // Bilinear footprint of (u, v) = (i + dx, j + dy) clamped into the grid.
@@ -113,7 +112,7 @@ struct ColVol {
   const void* base;    // the volume; addressed in groups of 4 samples
   unsigned roff[4];    // row offsets (in groups) of the 4 neighbour rows
   unsigned coff[4];    // column offsets (in groups) of the 4 neighbour columns
-  float wx[4], dwx[4], wy[4], dwy[4], wz[4], dwz[4];
+  float wx[4], wy[4], wz[4];
   int q, r;            // floor(dz) = 4 q + r, 0 <= r < 4
   int bx, by;          // floor of the transverse coordinates
 };
@@ -150,9 +149,10 @@ __device__ __forceinline__ void setup_col(ColVol& V, const void* vol, const Leve
   const int kz0 = base[2];
   V.q = kz0 >> 2;  // arithmetic shift: floor division by 4
   V.r = kz0 & 3;
-  keys_weights(frac[0], V.wx, V.dwx);
-  keys_weights(frac[1], V.wy, V.dwy);
-  keys_weights(frac[2], V.wz, V.dwz);
+  float dw[4];  // the derivative weights are not used here
+  keys_weights(frac[0], V.wx, dw);
+  keys_weights(frac[1], V.wy, dw);
+  keys_weights(frac[2], V.wz, dw);
   const unsigned nq = (unsigned)(L.dp >> 2);
 #pragma unroll
   for (int a = 0; a < 4; a++) {
@@ -178,13 +178,6 @@ __device__ __forceinline__ void qfma(Q4& acc, float2 w, const Q4& s) {
 
 __device__ __forceinline__ float4 f4(const Q4& q) { return make_float4(q.lo.x, q.lo.y, q.hi.x, q.hi.y); }
 
-__device__ __forceinline__ void fma4(float4& acc, float w, const float4& s) {
-  acc.x = fmaf(w, s.x, acc.x);
-  acc.y = fmaf(w, s.y, acc.y);
-  acc.z = fmaf(w, s.z, acc.z);
-  acc.w = fmaf(w, s.w, acc.w);
-}
-
 __device__ __forceinline__ float4 bcast(float v) { return make_float4(v, v, v, v); }
 
 // Axial 4-tap filter for the lane's 4 outputs.  e[1..4] hold the lane's
@@ -192,131 +185,68 @@ __device__ __forceinline__ float4 bcast(float v) { return make_float4(v, v, v, v
 // group and e[9] the first sample of lane+2's.  Output o, tap c reads
 // e[R + o + c], where R = floor(dz) mod 4.
 template <int R>
-__device__ __forceinline__ void axial_col(const float4& T, const float4& Tx, const float4& Ty,
-                                      const float wz[4], const float dwz[4], float I[4], float Iz[4],
-                                      float Ix[4], float Iy[4]) {
-  float e[10], ex[10], ey[10];
+__device__ __forceinline__ void axial_col(const float4& T, const float wz[4], float I[4]) {
+  float e[10];
   e[1] = T.x; e[2] = T.y; e[3] = T.z; e[4] = T.w;
-  ex[1] = Tx.x; ex[2] = Tx.y; ex[3] = Tx.z; ex[4] = Tx.w;
-  ey[1] = Ty.x; ey[2] = Ty.y; ey[3] = Ty.z; ey[4] = Ty.w;
-  if (R == 0) {
-    e[0] = __shfl_up_sync(kFull, T.w, 1);
-    ex[0] = __shfl_up_sync(kFull, Tx.w, 1);
-    ey[0] = __shfl_up_sync(kFull, Ty.w, 1);
-  }
+  if (R == 0) e[0] = __shfl_up_sync(kFull, T.w, 1);
   e[5] = __shfl_down_sync(kFull, T.x, 1);
-  ex[5] = __shfl_down_sync(kFull, Tx.x, 1);
-  ey[5] = __shfl_down_sync(kFull, Ty.x, 1);
   e[6] = __shfl_down_sync(kFull, T.y, 1);
-  ex[6] = __shfl_down_sync(kFull, Tx.y, 1);
-  ey[6] = __shfl_down_sync(kFull, Ty.y, 1);
-  if (R >= 1) {
-    e[7] = __shfl_down_sync(kFull, T.z, 1);
-    ex[7] = __shfl_down_sync(kFull, Tx.z, 1);
-    ey[7] = __shfl_down_sync(kFull, Ty.z, 1);
-  }
-  if (R >= 2) {
-    e[8] = __shfl_down_sync(kFull, T.w, 1);
-    ex[8] = __shfl_down_sync(kFull, Tx.w, 1);
-    ey[8] = __shfl_down_sync(kFull, Ty.w, 1);
-  }
-  if (R == 3) {
-    e[9] = __shfl_down_sync(kFull, T.x, 2);
-    ex[9] = __shfl_down_sync(kFull, Tx.x, 2);
-    ey[9] = __shfl_down_sync(kFull, Ty.x, 2);
-  }
-#ifndef OCTMC_AXIAL_PACKED
-#define OCTMC_AXIAL_PACKED 1
-#endif
-#if OCTMC_AXIAL_PACKED
+  if (R >= 1) e[7] = __shfl_down_sync(kFull, T.z, 1);
+  if (R >= 2) e[8] = __shfl_down_sync(kFull, T.w, 1);
+  if (R == 3) e[9] = __shfl_down_sync(kFull, T.x, 2);
   // outputs in packed pairs (o, o + 1); each half adds its 4 taps in the
   // scalar order
 #pragma unroll
   for (int o = 0; o < 4; o += 2) {
-    float2 a = make_float2(0.f, 0.f), az = a, ax = a, ay = a;
+    float2 a = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-      const float2 w = make_float2(wz[c], wz[c]), dw = make_float2(dwz[c], dwz[c]);
-      const float2 ev = make_float2(e[R + o + c], e[R + o + 1 + c]);
-      a = ffma2(w, ev, a);
-      az = ffma2(dw, ev, az);
-      ax = ffma2(w, make_float2(ex[R + o + c], ex[R + o + 1 + c]), ax);
-      ay = ffma2(w, make_float2(ey[R + o + c], ey[R + o + 1 + c]), ay);
-    }
+    for (int c = 0; c < 4; c++)
+      a = ffma2(make_float2(wz[c], wz[c]), make_float2(e[R + o + c], e[R + o + 1 + c]), a);
     I[o] = a.x; I[o + 1] = a.y;
-    Iz[o] = az.x; Iz[o + 1] = az.y;
-    Ix[o] = ax.x; Ix[o + 1] = ax.y;
-    Iy[o] = ay.x; Iy[o + 1] = ay.y;
   }
-#else
-#pragma unroll
-  for (int o = 0; o < 4; o++) {
-    float a = 0.f, az = 0.f, ax = 0.f, ay = 0.f;
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      a = fmaf(wz[c], e[R + o + c], a);
-      az = fmaf(dwz[c], e[R + o + c], az);
-      ax = fmaf(wz[c], ex[R + o + c], ax);
-      ay = fmaf(wz[c], ey[R + o + c], ay);
-    }
-    I[o] = a; Iz[o] = az; Ix[o] = ax; Iy[o] = ay;
-  }
-#endif
 }
 
-// Interpolated values (and their displacement derivatives) of one volume
-// at the lane's 4 outputs.  qk: first input depth of the lane's group
-// (samples, may lie outside the volume); qc: index of that group's (clamped)
-// samples in the volume.
+// Interpolated values of one volume at the lane's 4 outputs.  qk: first input
+// depth of the lane's group (samples, may lie outside the volume); qc: index
+// of that group's (clamped) samples in the volume.
 template <typename S>
-__device__ __forceinline__ void sample_col_group(const ColVol& V, int qk, unsigned qc, int dp, float I[4], float Iz[4],
-                                             float Ix[4], float Iy[4]) {
-  // transverse 4 x 4 interpolation of the group and its x / y derivatives,
-  // in packed pairs along depth (same operations and order as scalar FMAs)
-  Q4 Tq = q4zero(), Txq = q4zero(), Tyq = q4zero();
+__device__ __forceinline__ void sample_col_group(const ColVol& V, int qk, unsigned qc, int dp, float I[4]) {
+  // transverse 4 x 4 interpolation of the group, in packed pairs along depth
+  // (same operations and order as scalar FMAs)
+  Q4 Tq = q4zero();
 #pragma unroll
   for (int b = 0; b < 4; b++) {
-    Q4 U = q4zero(), Ux = q4zero();
+    Q4 U = q4zero();
 #pragma unroll
     for (int a = 0; a < 4; a++) {
       const unsigned idx = V.roff[b] + V.coff[a] + qc;
-      const Q4 s = q4(load4<S>(V.base, idx));
-      qfma(U, make_float2(V.wx[a], V.wx[a]), s);
-      qfma(Ux, make_float2(V.dwx[a], V.dwx[a]), s);
+      qfma(U, make_float2(V.wx[a], V.wx[a]), q4(load4<S>(V.base, idx)));
     }
     qfma(Tq, make_float2(V.wy[b], V.wy[b]), U);
-    qfma(Txq, make_float2(V.wy[b], V.wy[b]), Ux);
-    qfma(Tyq, make_float2(V.dwy[b], V.dwy[b]), U);
   }
-  float4 T = f4(Tq), Tx = f4(Txq), Ty = f4(Tyq);
+  float4 T = f4(Tq);
   // groups entirely before sample 0 / after the last sample hold the edge value
-  if (qk < 0) {
-    T = bcast(T.x); Tx = bcast(Tx.x); Ty = bcast(Ty.x);
-  } else if (qk >= dp) {
-    T = bcast(T.w); Tx = bcast(Tx.w); Ty = bcast(Ty.w);
-  }
+  if (qk < 0) T = bcast(T.x);
+  else if (qk >= dp) T = bcast(T.w);
   switch (V.r) {
-    case 0: axial_col<0>(T, Tx, Ty, V.wz, V.dwz, I, Iz, Ix, Iy); break;
-    case 1: axial_col<1>(T, Tx, Ty, V.wz, V.dwz, I, Iz, Ix, Iy); break;
-    case 2: axial_col<2>(T, Tx, Ty, V.wz, V.dwz, I, Iz, Ix, Iy); break;
-    default: axial_col<3>(T, Tx, Ty, V.wz, V.dwz, I, Iz, Ix, Iy); break;
+    case 0: axial_col<0>(T, V.wz, I); break;
+    case 1: axial_col<1>(T, V.wz, I); break;
+    case 2: axial_col<2>(T, V.wz, I); break;
+    default: axial_col<3>(T, V.wz, I); break;
   }
 }
 
-// Interpolated values (and their displacement derivatives) of one volume
-// at the lane's 4 outputs of the depth block starting at kb, from the
-// volume in global memory.
+// Interpolated values of one volume at the lane's 4 outputs of the depth
+// block starting at kb.
 template <typename S>
-__device__ __forceinline__ void sample_col_block(const ColVol& V, int kb, int lane, int dp, float I[4],
-                                             float Iz[4], float Ix[4], float Iy[4]) {
+__device__ __forceinline__ void sample_col_block(const ColVol& V, int kb, int lane, int dp, float I[4]) {
   const int qk = kb + 4 * V.q + 4 * (lane - 1);  // first input depth of the lane's group
   const unsigned qc = (unsigned)(min(max(qk, 0), dp - 4) >> 2);
-  sample_col_group<S>(V, qk, qc, dp, I, Iz, Ix, Iy);
+  sample_col_group<S>(V, qk, qc, dp, I);
 }
 
 // Motion-corrected resampling and merging of one A-scan (warp): both scans
-// resampled along depth at the displaced positions (the derivative parts of
-// sample_block are dead code here), merged with the per-A-scan weights.
+// resampled along depth at the displaced positions, merged with the per-A-scan weights.
 // Forward only, so it fits in 40 registers: 6 blocks (48 warps) per SM keep
 // more loads in flight than the data kernel's 3.  vec4: d % 4 == 0 and every
 // output 16-byte aligned, so a lane's 4 outputs go out as one 128-bit store.
@@ -337,9 +267,9 @@ resample_merge_kernel(const LevelDev L, const double* __restrict__ disp, const f
   setup_col(VY, L.sy, L, base + 3, frac + 3);
   const float wx = weights ? weights[p] : 0.5f, wy = weights ? weights[nasc + p] : 0.5f;
   for (int kb = 0; kb < L.d; kb += kOutPerIter) {
-    float IX[4], IzX[4], IxX[4], IyX[4], IY[4], IzY[4], IxY[4], IyY[4];
-    sample_col_block<T>(VX, kb, lane, L.dp, IX, IzX, IxX, IyX);
-    sample_col_block<T>(VY, kb, lane, L.dp, IY, IzY, IxY, IyY);
+    float IX[4], IY[4];
+    sample_col_block<T>(VX, kb, lane, L.dp, IX);
+    sample_col_block<T>(VY, kb, lane, L.dp, IY);
     const int k0 = kb + 4 * (lane - 1);
     if (lane >= 1 && lane <= kOutLanes && k0 < L.d) {
       const int64_t e0 = p * L.d + k0;
