@@ -84,8 +84,9 @@ class BatchObjectiveFunction(torch.autograd.Function):
         else:
             grads = [torch.empty_like(D) for D in saved]
             eval_batch(ctx.problems, [ctx.level] * len(saved), list(saved), grads)
-        # one launch for the whole batch
-        return (None, None, None) + tuple(torch._foreach_mul(grads, grad_out.to(grads[0].dtype)))
+        # one product per gradient: torch._foreach_mul takes one launch for all (8 gradients of 128 x 128: 54 us
+        # against 94 us) but has no batching rule and fails under is_grads_batched and create_graph
+        return (None, None, None) + tuple(grad_out.to(g.dtype) * g for g in grads)
 
 
 def batch_objective(problems, level, disps, mode="recompute"):
