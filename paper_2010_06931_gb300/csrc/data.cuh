@@ -14,17 +14,18 @@ namespace {
 
 // Eq. 4 (or squared differences) of a residual and its derivative.  The
 // pseudo-Huber loss is evaluated as (R^2/eps) / (1 + sqrt(1 + (R/eps)^2)): no
-// cancellation near 0.  Its arguments are never subnormal (1 + x^2 >= 1), so
-// the flush-to-zero forms of the reciprocal square root and the division give
-// the same results without the scaling of subnormals.
+// cancellation near 0.  The square root's argument is at least 1 and the
+// divisor between 1 and 2^65, so neither of their flush-to-zero approximations
+// meets a subnormal, and they save its scaling.  The numerator R^2/eps can be
+// subnormal: it is multiplied by the divisor's reciprocal without flushing.
 __device__ __forceinline__ float rsqrt_ge1(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ float div_ge1(float a, float b) {
+__device__ __forceinline__ float rcp_ge1(float x) {
   float y;
-  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 __device__ __forceinline__ void loss_grad(float R, float inv_eps, bool ssd, float* Lv, float* dL) {
@@ -36,7 +37,7 @@ __device__ __forceinline__ void loss_grad(float R, float inv_eps, bool ssd, floa
     const float qv = fmaf(rr, rr, 1.0f);
     const float is = rsqrt_ge1(qv);
     *dL = rr * is;
-    *Lv = div_ge1(R * rr, fmaf(qv, is, 1.0f));
+    *Lv = __fmul_rn(R * rr, rcp_ge1(fmaf(qv, is, 1.0f)));
   }
 }
 
