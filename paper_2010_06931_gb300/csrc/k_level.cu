@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kLThreads, 1) level_kernel(const __grid_consta
   __shared__ unsigned long long s_gmax;
   __shared__ const double* s_hp[kMaxVec];
   __shared__ double s_cf[kMaxVec];
-  __shared__ VolTab tab[kLWarps][2];
+  __shared__ VolTab tab[kLWarps][2][2];  // per warp two pairs, taken in turn (eval_ascan)
   copy_state<kLThreads, sizeof(SolveState)>(&sS, A.S);
   __syncthreads();
   const int G = gridDim.x, B = blockIdx.x;
@@ -225,8 +225,9 @@ __global__ void __launch_bounds__(kLThreads, 1) level_kernel(const __grid_consta
       double acc[4] = {0.0, 0.0, 0.0, 0.0};  // S^str, S^ang, R, grad . dir
       unsigned long long gmx = 0ull;
       const float two_mu_s = (float)(2.0 * A.mu * s_ms[lane < 6 ? lane % 3 : 0]);
-      for (int64_t p = (int64_t)B * kLWarps + warp; p < plane; p += (int64_t)G * kLWarps)
-        eval_ascan<T>(A.D, tab[warp], V.gt, V.dir, p, lane, two_mu_s, inv_eps_r, alpha_d, acc, &gmx);
+      int turn = 0;
+      for (int64_t p = (int64_t)B * kLWarps + warp; p < plane; p += (int64_t)G * kLWarps, turn ^= 1)
+        eval_ascan<T>(A.D, tab[warp][turn], V.gt, V.dir, p, lane, two_mu_s, inv_eps_r, alpha_d, acc, &gmx);
       lblock_sum<4>(acc);
       gmx = lblock_max(gmx);
       if (tid == 0) {

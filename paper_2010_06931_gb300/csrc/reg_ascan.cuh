@@ -19,14 +19,19 @@ __device__ __forceinline__ float huber_r(float x, float inv_eps, float* dl) {
   return __fdividef(x * r, fmaf(q, is, 1.0f));
 }
 
-// One A-scan of the evaluation by one warp: the data term (lanes 0..7 hold
-// its outputs), then lanes 0..5 the regulariser terms, the mean-term
+// One A-scan of the evaluation by one warp: the data term (lane 4 v holds
+// its output v), then lanes 0..5 the regulariser terms, the mean-term
 // gradient and the float64 gradient of component 3 V + c = lane; partial
 // sums into acc (S^str, S^ang, R, grad . dir) and the running max |grad|.
+// A warp that takes one A-scan after another alternates between two tables:
+// between an A-scan's last read of a table and the next write to it then lies
+// the warp barrier after the other table's writes (setup_pair).  One table and
+// a second barrier per A-scan instead spills 1068 bytes at the level kernel's
+// 64 registers (388 with two tables).
 template <typename T>
-__device__ __forceinline__ void eval_ascan(const DataArgs& D, VolTab* tab, double* __restrict__ grad, const double* __restrict__ dir,
-                                           int64_t p, int lane, float two_mu_s, float inv_eps_r, float alpha_d,
-                                           double* acc, unsigned long long* gmx) {
+__device__ __forceinline__ void eval_ascan(const DataArgs& D, VolTab* tab, double* __restrict__ grad,
+                                           const double* __restrict__ dir, int64_t p, int lane, float two_mu_s,
+                                           float inv_eps_r, float alpha_d, double* acc, unsigned long long* gmx) {
   const LevelDev& L = D.L;
   const int64_t plane = (int64_t)L.w * L.h;
   const double* xt = D.disp;
