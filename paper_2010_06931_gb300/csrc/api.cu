@@ -304,7 +304,7 @@ struct octmc_problem {
   bool have_ang = false;
   std::vector<Level> lv;
   char* slab = nullptr;       // one allocation: the levels and the evaluation workspace
-  char* build_tmp = nullptr;  // buffers of the construction
+  char* build_tmp = nullptr;  // float32 volumes of the construction (16-bit storage)
   // evaluation workspace (sized for level 0)
   float* str = nullptr;
   float* ang = nullptr;
@@ -441,8 +441,18 @@ struct BuildTemps {
   ChainInfo* info = nullptr;    // [level][scan]
 };
 
-// Every buffer a problem keeps, level by level, and the evaluation workspace.
-void lay_out(octmc_problem* P, Arena& A) {
+// The sampling times and the chains' test of every level.
+void lay_out_times(octmc_problem* P, BuildTemps& B, Arena& A) {
+  for (int V = 0; V < 2; V++) {
+    B.t[V].clear();
+    for (const Level& Lv : P->lv) B.t[V].push_back(A.take<double>((size_t)Lv.dev.w * Lv.dev.h));
+  }
+  B.info = A.take<ChainInfo>(2 * P->lv.size());
+}
+
+// Every buffer a problem keeps, level by level, and the evaluation workspace,
+// whose float gradient lies where the construction had the sampling times.
+void lay_out(octmc_problem* P, BuildTemps& B, Arena& A) {
   const octmc_desc& D = P->desc;
   int w = D.w, h = D.h, d = D.d;
   for (int l = 0; l < D.levels; l++) {
@@ -472,23 +482,24 @@ void lay_out(octmc_problem* P, Arena& A) {
   const int64_t n0 = P->plane(0);
   P->str = A.take<float>((size_t)n0);
   P->ang = A.take<float>((size_t)n0);
-  P->gdata = A.take<float>((size_t)6 * n0);
+  Arena T{A.base ? A.base + A.used : nullptr, 0};
+  lay_out_times(P, B, T);
+  P->gdata = reinterpret_cast<float*>(A.take<char>(std::max(T.used, sizeof(float) * 6 * (size_t)n0)));
   P->partials = A.take<double>((size_t)8 * std::max(reg_grid_blocks(n0), msum_grid_blocks()));
   P->counters = A.take<unsigned>(2);
   P->res = A.take<EvalResult>(1);
 }
 
-void lay_out_temps(octmc_problem* P, BuildTemps& B, Arena& A) {
-  B.vol[0].clear(); B.vol[1].clear(); B.t[0].clear(); B.t[1].clear();
-  for (const Level& Lv : P->lv) {
-    const LevelDev& X = Lv.dev;
-    const size_t cols = (size_t)X.w * X.h;
-    for (int V = 0; V < 2; V++) {
-      B.vol[V].push_back(X.dtype == OCTMC_F32 ? static_cast<float*>(V == 0 ? X.sx : X.sy) : A.take<float>(cols * X.dp));
-      B.t[V].push_back(A.take<double>(cols));
+// The float32 volumes: temporaries with 16-bit storage.
+void lay_out_volumes(octmc_problem* P, BuildTemps& B, Arena& A) {
+  for (int V = 0; V < 2; V++) {
+    B.vol[V].clear();
+    for (const Level& Lv : P->lv) {
+      const LevelDev& X = Lv.dev;
+      B.vol[V].push_back(X.dtype == OCTMC_F32 ? static_cast<float*>(V == 0 ? X.sx : X.sy)
+                                              : A.take<float>((size_t)X.w * X.h * X.dp));
     }
   }
-  B.info = A.take<ChainInfo>(2 * P->lv.size());
 }
 
 // The chain of one scan by a sort on the host: times in neither raster order.
@@ -506,28 +517,35 @@ void host_chain(octmc_problem* P, const double* t_dev, const LevelDev& X, int V)
   CK(cudaStreamSynchronize(P->st));  // host vectors go out of scope
 }
 
-// Everything a problem keeps lives in one allocation, and everything that only
-// its construction needs in a second one; the work is enqueued without a host
-// wait until the chains' test is read at the end.  300 x 300 x 512, 3 levels,
-// device inputs: 9.8 -> 1.44 ms with its destruction.
+// Everything a problem keeps lives in one allocation; with 16-bit storage the
+// float32 volumes that only its construction needs live in a second one.
+// float32 storage frees nothing here: cudaFree waits for the whole device, so
+// a problem created beside running solves would wait for them (an admission to
+// the server beside a solve of 151 ms: 151 ms with a second allocation for the
+// sampling times, freed at the end, 0.5 ms without).  The work is enqueued
+// without a host wait until the chains' test is read at the end.
+// 300 x 300 x 512, 3 levels, device inputs: 9.8 -> 1.33 ms with its destruction.
 void create_impl(octmc_problem* P) {
   const octmc_desc& D = P->desc;
   check_device();
   const int L = D.levels;
   const int dt = D.storage;
   P->lv.resize(L);
-  Arena size, keep, tmp;
-  lay_out(P, size);
+  BuildTemps B;
+  Arena size;
+  lay_out(P, B, size);
   P->slab = dalloc<char>(size.used);
-  keep.base = P->slab;
-  lay_out(P, keep);
+  Arena keep{P->slab, 0};
+  lay_out(P, B, keep);
   // The pyramid is built in float32; with 16-bit storage every level is
   // rounded once (to nearest even) from its float32 box means.
-  BuildTemps B;
-  lay_out_temps(P, B, tmp);
-  P->build_tmp = dalloc<char>(tmp.used);
-  tmp = Arena{P->build_tmp, 0};
-  lay_out_temps(P, B, tmp);
+  if (dt != OCTMC_F32) {
+    Arena tsize;
+    lay_out_volumes(P, B, tsize);
+    P->build_tmp = dalloc<char>(tsize.used);
+  }
+  Arena tmp{P->build_tmp, 0};
+  lay_out_volumes(P, B, tmp);
   CK(cudaMemsetAsync(P->counters, 0, 2 * sizeof(unsigned), P->st));
   std::vector<ChainInfo> info(2 * L);
   const ChainInfo none{0, 0, 0, 0, 0x7ff0000000000000ull, 0x7ff0000000000000ull};
