@@ -297,8 +297,8 @@ int octmc_enface_ws(const float *octa_dev, const float *oct_dev, int w, int h, i
                     const float *v_dev, double q_lo, double q_hi, double thresh, double t_oct, float *enface_dev,
                     float *filtered_dev, double *info_host, void *workspace_dev, int64_t workspace_bytes,
                     void *stream);
-/* Bytes of scratch octmc_enface_ws needs for a scan of this size; -1 for an
- * invalid size. */
+/* Bytes of scratch octmc_enface_ws needs for a scan of this size; -1 for a
+ * size that it refuses. */
 int64_t octmc_enface_workspace(int w, int h, int d, int fast_axis);
 
 /* Copies pyramid data of `level` to device buffers (any may be NULL):

@@ -738,15 +738,20 @@ struct EnfaceScratch {
   }
 };
 
+// Whether a projection takes scans of this size.
+int enface_size(int w, int h, int d, int fast_axis) {
+  if (w < 1 || h < 1 || d < 1 || (fast_axis != 0 && fast_axis != 1)) return OCTMC_ERR_INVALID_ARG;
+  const int nf = fast_axis == 0 ? w : h;
+  return nf > kMaxFast || h > 65535 || (w + 7) / 8 > 65535 ? OCTMC_ERR_UNSUPPORTED : OCTMC_OK;
+}
+
 int enface_check(const float* octa, const float* oct, int w, int h, int d, int fast_axis, const float* v, double q_lo,
                  double q_hi, double thresh, const float* enface) {
-  if (!octa || !oct || !v || !enface || w < 1 || h < 1 || d < 1 || (fast_axis != 0 && fast_axis != 1))
-    return OCTMC_ERR_INVALID_ARG;
+  const int size = enface_size(w, h, d, fast_axis);
+  if (!octa || !oct || !v || !enface || size == OCTMC_ERR_INVALID_ARG) return OCTMC_ERR_INVALID_ARG;
   if (!(q_lo >= 0.0 && q_lo <= 1.0 && q_hi >= 0.0 && q_hi <= 1.0) || !std::isfinite(thresh))
     return OCTMC_ERR_INVALID_ARG;
-  const int nf = fast_axis == 0 ? w : h;
-  if (nf > kMaxFast || h > 65535 || (w + 7) / 8 > 65535) return OCTMC_ERR_UNSUPPORTED;
-  return OCTMC_OK;
+  return size;
 }
 
 void rank15(const float* in, int w, int h, int d, int axis, float* out, cudaStream_t st) {
@@ -851,7 +856,7 @@ extern "C" int octmc_saccade_validity(const float* octa, int w, int h, int d, in
 }
 
 extern "C" int64_t octmc_enface_workspace(int w, int h, int d, int fast_axis) {
-  if (w < 1 || h < 1 || d < 1 || (fast_axis != 0 && fast_axis != 1)) return -1;
+  if (enface_size(w, h, d, fast_axis) != OCTMC_OK) return -1;
   return (int64_t)EnfaceScratch(nullptr, (int64_t)w * h * d, fast_axis == 0 ? h : w).bytes;
 }
 
