@@ -133,22 +133,6 @@ __device__ __forceinline__ double widen_exact(float x) {
   return __hiloint2double((int)hi, (int)lo);
 }
 
-// Double to float by truncating the mantissa (integer instructions only):
-// values below the float normal range become signed zero, values beyond it
-// infinity; NaN stays NaN.
-__device__ __forceinline__ float narrow_trunc(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned h = (unsigned)(b >> 32);
-  const unsigned sign = h & 0x80000000u;
-  const int e = (int)((h >> 20) & 0x7ffu);
-  const unsigned mant = (unsigned)((b >> 29) & 0x7fffffu);
-  if (e == 0x7ff) return __uint_as_float(sign | 0x7f800000u | (mant | ((b & 0xFFFFFFFFFFFFFull) ? 1u : 0u)));
-  const int ef = e - 1023 + 127;
-  if (ef <= 0) return __uint_as_float(sign);
-  if (ef >= 255) return __uint_as_float(sign | 0x7f800000u);
-  return __uint_as_float(sign | ((unsigned)ef << 23) | mant);
-}
-
 // The exact sum of 8 floats as s + e, s the rounded sum (Knuth's two-sum).
 // Float64 additions run at 1/64 of the float rate on this GPU; this takes 42
 // float additions for 8.  True where the sum is exact: the non-zero magnitudes
@@ -315,16 +299,14 @@ struct RegArgs {
 };
 
 // Batched evaluation of several problems ("slots") in one launch per
-// kernel.  Data kernel: slot s owns the A-scans [begin[s], begin[s+1]) of
-// the launch.  Reduction kernels: slot s owns the blocks [b0[s], b0[s+1]) --
-// the same number and partition of blocks as a launch for that slot alone,
-// so its sums do not depend on the other slots.  The arguments travel in the
-// kernel parameter block (at most 32 KB).
+// kernel.  Data kernel: grid (tiles, slots), slot s owns row s of the grid.
+// Reduction kernels: slot s owns the blocks [b0[s], b0[s+1]) -- the same
+// number and partition of blocks as a launch for that slot alone, so its sums
+// do not depend on the other slots.  The arguments travel in the kernel
+// parameter block (at most 32 KB).
 constexpr int kMaxSlots = 48;
 struct DataMulti {
   int nslots;
-  int64_t total;
-  int64_t begin[kMaxSlots + 1];
   DataArgs da[kMaxSlots];
 };
 struct MsumSlot {

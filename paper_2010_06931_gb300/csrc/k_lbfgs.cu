@@ -201,14 +201,13 @@ int hist_dots_blocks(int64_t n) {
 
 cudaError_t launch_hist_dots(const HistDots& hd, int64_t n, double* partials, unsigned* counter, double* out,
                              cudaStream_t s) {
-  if (hd.K < 0 || hd.K > kMaxHist) return cudaErrorInvalidValue;
+  if (hd.K < 0 || hd.K > kMaxHist || (!hd.q0 && !hd.q1)) return cudaErrorInvalidValue;
   const int G = hist_dots_blocks(n);
   const int rows = hd.K > 0 ? (hd.K + kHistChunk - 1) / kHistChunk : 1;
   const dim3 g(G, rows);
   if (hd.q0 && hd.q1) hist_dots_kernel<true, true><<<g, kThreads, 0, s>>>(hd, n, partials, counter, out);
   else if (hd.q0) hist_dots_kernel<true, false><<<g, kThreads, 0, s>>>(hd, n, partials, counter, out);
-  else if (hd.q1) hist_dots_kernel<false, true><<<g, kThreads, 0, s>>>(hd, n, partials, counter, out);
-  else hist_dots_kernel<false, false><<<g, kThreads, 0, s>>>(hd, n, partials, counter, out);
+  else hist_dots_kernel<false, true><<<g, kThreads, 0, s>>>(hd, n, partials, counter, out);
   return cudaGetLastError();
 }
 
