@@ -35,29 +35,6 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
   return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
 
-// Reduce-scatter of 2 N per-lane float64 values over the lanes paired by bit N
-// (see warp_reduce_scatter32): a lane does 31 float64 additions for 32 sums
-// where a butterfly per sum would do 160.
-template <int N>
-__device__ __forceinline__ void rs_stage(double* v, int lane) {
-  const bool up = (lane & N) != 0;
-#pragma unroll
-  for (int j = 0; j < N; j++) {
-    const double send = up ? v[j] : v[j + N];
-    const double keep = up ? v[j + N] : v[j];
-    v[j] = keep + __shfl_xor_sync(0xffffffffu, send, N);
-  }
-}
-// v[0] of lane i becomes the warp total of value i.
-__device__ __forceinline__ double warp_reduce_scatter32(double* v, int lane) {
-  rs_stage<16>(v, lane);
-  rs_stage<8>(v, lane);
-  rs_stage<4>(v, lane);
-  rs_stage<2>(v, lane);
-  rs_stage<1>(v, lane);
-  return v[0];
-}
-
 // grid (G, rows): block (bx, r) takes history vectors r*6 .. r*6+5 over
 // a contiguous share of the n elements; row 0 also takes
 // q0.q0, q1.q1 and max|q1| (the maximum on the bit patterns: exact, and NaN

@@ -151,32 +151,6 @@ __global__ void __launch_bounds__(kThreads) finish_kernel(const SolveState* __re
     V.x[e] = xs[e];
 }
 
-// Reduce-scatter of 32 per-lane float64 values over the warp: on return v[0]
-// of lane i is the warp total of value i.  Each stage keeps half of the
-// values and adds the partner lane's copy of that half, so a lane does 31
-// float64 adds for 32 values (a butterfly per value would do 160, and this
-// GPU runs float64 at 1/64 of the float rate).  The pairing is fixed, so the
-// sums are reproducible.
-template <int N>
-__device__ __forceinline__ void rs_stage(double* v, int lane) {
-  const bool up = (lane & N) != 0;
-#pragma unroll
-  for (int j = 0; j < N; j++) {
-    const double send = up ? v[j] : v[j + N];
-    const double keep = up ? v[j + N] : v[j];
-    v[j] = keep + __shfl_xor_sync(0xffffffffu, send, N);
-  }
-}
-
-__device__ __forceinline__ double warp_reduce_scatter32(double* v, int lane) {
-  rs_stage<16>(v, lane);
-  rs_stage<8>(v, lane);
-  rs_stage<4>(v, lane);
-  rs_stage<2>(v, lane);
-  rs_stage<1>(v, lane);
-  return v[0];
-}
-
 // The products pass over this block's share of the elements, with gp the
 // gradient at the iterate the products are for.  After an accepted step the
 // new pair s = xs - x, y = gp - g is formed here; the row whose candidates
