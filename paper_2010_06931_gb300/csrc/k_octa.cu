@@ -267,7 +267,59 @@ __device__ __forceinline__ float median27(const Slab& A, const Slab& B, const Sl
   return median3_of(a[4], a[5], a[6]);
 }
 
+// The median of 27 samples some of which may be NaN: a minimum or maximum of a
+// NaN and a number is the number, so which numbers take the NaNs' places
+// depends on the order of the exchanges.  This order defines it: the 9 columns
+// r[0..2] + o[0..2] sorted along depth, then the 13 values that median27 keeps
+// by partial selection over the 9 lows, mids and highs.
+__device__ __forceinline__ float median27_nan(const float* const r[3], const int64_t o[3], int km, int kp) {
+  float lo[9], mid[9], hi[9];
+#pragma unroll
+  for (int c = 0; c < 9; c++) {
+    const float* col = r[c / 3] + o[c % 3];
+    lo[c] = __ldg(col + km);
+    mid[c] = __ldg(col);
+    hi[c] = __ldg(col + kp);
+    sort3(lo[c], mid[c], hi[c]);
+  }
+#pragma unroll
+  for (int e = 8; e >= 5; e--)  // the 4 largest lows
+#pragma unroll
+    for (int i = 0; i < e; i++) cmpx(lo[i], lo[e]);
+#pragma unroll
+  for (int b = 0; b <= 3; b++)  // the 4 smallest highs
+#pragma unroll
+    for (int i = b + 1; i < 9; i++) cmpx(hi[b], hi[i]);
+#pragma unroll
+  for (int q = 0; q < 2; q++) {  // the middle 5 mids
+    cmpx(mid[q], mid[8 - q]);
+#pragma unroll
+    for (int i = q + 1; i < 8 - q; i++) {
+      cmpx(mid[q], mid[i]);
+      cmpx(mid[i], mid[8 - q]);
+    }
+  }
+  float a[8] = {lo[5], lo[6], lo[7], lo[8], mid[2], mid[3], mid[4], mid[5]};
+  const float rest[5] = {mid[6], hi[0], hi[1], hi[2], hi[3]};
+  forget_steps<8, 5>(a, rest);
+  return median3_of(a[5], a[6], a[7]);
+}
+
 constexpr int kSx = 32, kSy = 8;
+
+// The medians of columns i0..i0+n-1 at (j, k) where a sample may be NaN.  Out
+// of line: strips of numbers never come here.
+__device__ __noinline__ void median_strip_nan(const float* __restrict__ in, int w, int h, int d, int i0, int n, int j,
+                                              int k, float* __restrict__ out) {
+  const int64_t row = (int64_t)w * d;
+  const float* r[3] = {in + clampn(j - 1, h) * row + k, in + j * row + k, in + clampn(j + 1, h) * row + k};
+  const int km = k > 0 ? -1 : 0, kp = k + 1 < d ? 1 : 0;
+#pragma unroll 1
+  for (int i = i0; i < i0 + n; i++) {
+    const int64_t o[3] = {(int64_t)clampn(i - 1, w) * d, (int64_t)i * d, (int64_t)clampn(i + 1, w) * d};
+    out[j * row + o[1] + k] = median27_nan(r, o, km, kp);
+  }
+}
 
 // Block (32 depths, 8 strips), grid (depth chunks, groups of strips, rows): a
 // thread walks kMedI consecutive columns i of one row, so each slab's 18
@@ -285,15 +337,19 @@ __global__ void __launch_bounds__(kSx * kSy) median3_kernel(const float* __restr
   const int64_t row = (int64_t)w * d;
   const float* r[3] = {in + clampn(j - 1, h) * row + k, in + j * row + k, in + clampn(j + 1, h) * row + k};
   const int km = k > 0 ? -1 : 0, kp = k + 1 < d ? 1 : 0;
+  float sum = 0.f;  // of all samples: NaN if one of them is (or infinities of both signs are among them)
   auto slab = [&](int i, Slab& S) {
     const int64_t o = (int64_t)clampn(i, w) * d;
+    float part = 0.f;
 #pragma unroll
     for (int q = 0; q < 3; q++) {
       S.lo[q] = __ldg(r[q] + o + km);
       S.mid[q] = __ldg(r[q] + o);
       S.hi[q] = __ldg(r[q] + o + kp);
+      part += S.lo[q] + S.mid[q] + S.hi[q];
       sort3(S.lo[q], S.mid[q], S.hi[q]);
     }
+    sum += part;
     sort3(S.lo[0], S.lo[1], S.lo[2]);
     sort3(S.mid[0], S.mid[1], S.mid[2]);
     sort3(S.hi[0], S.hi[1], S.hi[2]);
@@ -309,6 +365,7 @@ __global__ void __launch_bounds__(kSx * kSy) median3_kernel(const float* __restr
     A = B;
     B = C;
   }
+  if (sum != sum) median_strip_nan(in, w, h, d, i0, n, j, k, out);
 }
 
 // The 3 smallest of a running set, sorted.
@@ -323,6 +380,20 @@ struct Low3 {
   }
 };
 
+// The outputs of one segment where a sample may be NaN: each window's samples
+// in turn.  A NaN repeats the smallest sample before it in the window, so the
+// split windows of rank15_kernel would give other values.
+constexpr int kSeg = 15, kRad = 7;
+__device__ __forceinline__ void rank_segment_nan(const float* c, int n, int64_t stride, int p0, float* o) {
+#pragma unroll 1
+  for (int u = 0; u < kSeg && p0 + u < n; u++) {
+    Low3 s = {INFINITY, INFINITY, INFINITY};
+#pragma unroll 1
+    for (int t = -kRad; t <= kRad; t++) s.add(__ldg(c + clampn(p0 + u + t, n) * stride));
+    o[u * stride] = s.c;
+  }
+}
+
 // 3rd smallest of the 15 samples p-7..p+7 along an axis.  A thread makes the 15
 // outputs of one segment at one depth: the windows split at the segment's
 // centre into a part of the 15 samples before and a part of the 14 after it, whose 3
@@ -331,7 +402,6 @@ struct Low3 {
 // loads instead of 75 and 15.  n, stride: length and stride of the axis; m,
 // ostride: the other transverse axis.  Bound by HBM and L2: 300 x 300 x 512
 // 100 us along x, 101 us along y (381 and 488 us one window per thread).
-constexpr int kSeg = 15, kRad = 7;
 __global__ void __launch_bounds__(kSx * kSy) rank15_kernel(const float* __restrict__ in, int n, int64_t stride, int m,
                                                            int64_t ostride, int d, float* __restrict__ out) {
   const int k = blockIdx.x * kSx + threadIdx.x;
@@ -341,9 +411,12 @@ __global__ void __launch_bounds__(kSx * kSy) rank15_kernel(const float* __restri
       const int p0 = seg * kSeg;
       const float* c = in + other * ostride + k;
       float* o = out + other * ostride + (int64_t)p0 * stride + k;
-      float x[kSeg];
+      float x[kSeg], sum = 0.f;  // sum: of all samples, as in median3_kernel
 #pragma unroll
-      for (int t = 0; t < kSeg; t++) x[t] = __ldg(c + clampn(p0 - kRad + t, n) * stride);
+      for (int t = 0; t < kSeg; t++) {
+        x[t] = __ldg(c + clampn(p0 - kRad + t, n) * stride);
+        sum += x[t];
+      }
       Low3 suf[kSeg];  // suf[t]: of x[t..14]
       suf[kSeg - 1] = {x[kSeg - 1], INFINITY, INFINITY};
 #pragma unroll
@@ -356,8 +429,13 @@ __global__ void __launch_bounds__(kSx * kSy) rank15_kernel(const float* __restri
       for (int u = 0; u < kSeg; u++) {
         if (p0 + u < n)
           o[u * stride] = fminf(fminf(suf[u].c, pre.c), fminf(fmaxf(suf[u].a, pre.b), fmaxf(suf[u].b, pre.a)));
-        if (u + 1 < kSeg) pre.add(__ldg(c + clampn(p0 + kRad + 1 + u, n) * stride));
+        if (u + 1 < kSeg) {
+          const float y = __ldg(c + clampn(p0 + kRad + 1 + u, n) * stride);
+          sum += y;
+          pre.add(y);
+        }
       }
+      if (sum != sum) rank_segment_nan(c, n, stride, p0, o);
     }
 }
 
