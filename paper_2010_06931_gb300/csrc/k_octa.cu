@@ -323,10 +323,11 @@ __device__ __noinline__ void median_strip_nan(const float* __restrict__ in, int 
 
 // Block (32 depths, 8 strips), grid (depth chunks, groups of strips, rows): a
 // thread walks kMedI consecutive columns i of one row, so each slab's 18
-// exchanges are made once for three medians, which then take 64 more (150 in
-// all when every voxel sorted its own 27 samples).  Bound by the minimum /
-// maximum rate (62 lanes per clock and SM measured): 300 x 300 x 512
-// 851 -> 442 us.
+// exchanges are made once for three medians, which then take 64 more: 86 per
+// voxel with the strips' ends (150 when every voxel sorted its own 27 samples).
+// Bound by the minimum / maximum rate (62 lanes per clock and SM measured; the
+// pipe is 90 % busy): 300 x 300 x 512 851 -> 454 us, with the sum that finds NaNs
+// taken per strip (a test per window costs 32 us more).
 constexpr int kMedI = 10;
 __global__ void __launch_bounds__(kSx * kSy) median3_kernel(const float* __restrict__ in, int w, int h, int d,
                                                             float* __restrict__ out) {
@@ -400,8 +401,9 @@ __device__ __forceinline__ void rank_segment_nan(const float* c, int n, int64_t 
 // smallest run along (5 minima / maxima per sample), and the 3rd smallest of
 // the two triples is min(s3, p3, max(s1, p2), max(s2, p1)): 15 per output and 2
 // loads instead of 75 and 15.  n, stride: length and stride of the axis; m,
-// ostride: the other transverse axis.  Bound by HBM and L2: 300 x 300 x 512
-// 100 us along x, 101 us along y (381 and 488 us one window per thread).
+// ostride: the other transverse axis.  Bound by the minimum / maximum rate (79 %
+// busy; HBM 48 %): 300 x 300 x 512 86 us along either axis (381 and 488 us one
+// window per thread; 100 us at the 70 registers it takes without the sum).
 __global__ void __launch_bounds__(kSx * kSy) rank15_kernel(const float* __restrict__ in, int n, int64_t stride, int m,
                                                            int64_t ostride, int d, float* __restrict__ out) {
   const int k = blockIdx.x * kSx + threadIdx.x;

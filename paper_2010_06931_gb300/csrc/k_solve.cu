@@ -202,7 +202,11 @@ __device__ __forceinline__ void dots_pass(const double* const* h, int kn, int cs
 // one-level solve with 6 / 10 / 14 vectors per row: 59.3 / 60.3 / 61.3 us
 // (64 x 64 x 64), 78.9 / 71.3 / 72.7 us (75 x 75 x 128), 151.4 / 142.2 / 146.2 us
 // (150 x 150 x 256): three rows of 6 need a second wave of blocks as soon as a
-// row has one block per SM.  Grid (G, rows): G blocks (one per SM) split the
+// row has one block per SM.  The same holds for rows of 10 from 10 pairs on:
+// 8 / 9 / 10 / 16 / 32 pairs 72.6 / 73.8 / 82.5 / 88.6 / 115.2 us (75 x 75 x 128)
+// and 549 / 548 / 597 / 596 / 671 us (300 x 300 x 512), 78.1 / 79.7 / 88.4 / 97.6 /
+// 136.0 and 649 / 649 / 699 / 702 / 794 us with rows of 20 at one block per SM
+// and the other kernels of that time.  Grid (G, rows): G blocks (one per SM) split the
 // elements into contiguous shares, rows cover the problem's longest history
 // (block (bx, r) takes candidates r*10 .. r*10+9; rows beyond this step's
 // candidates only arrive).  Within a block the float64 partial sums go
